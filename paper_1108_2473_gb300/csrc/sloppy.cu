@@ -270,67 +270,64 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-// fixed-order block reduction of two D4S (all ST threads participate)
-__device__ __forceinline__ void block_reduce_store2(D4S v0, D4S v1, D4S *dst0, D4S *dst1) {
-  __shared__ D4S sh[2][ST / 32];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  v0.a = warp_sum_d(v0.a);
-  v0.b = warp_sum_d(v0.b);
-  v0.c = warp_sum_d(v0.c);
-  v0.d = warp_sum_d(v0.d);
-  v1.a = warp_sum_d(v1.a);
-  v1.b = warp_sum_d(v1.b);
-  v1.c = warp_sum_d(v1.c);
-  v1.d = warp_sum_d(v1.d);
-  if (lane == 0) {
-    sh[0][w] = v0;
-    sh[1][w] = v1;
-  }
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    D4S t = sh[threadIdx.x][0];
-#pragma unroll
-    for (int k = 1; k < ST / 32; ++k) {
-      t.a += sh[threadIdx.x][k].a;
-      t.b += sh[threadIdx.x][k].b;
-      t.c += sh[threadIdx.x][k].c;
-      t.d += sh[threadIdx.x][k].d;
-    }
-    *(threadIdx.x ? dst1 : dst0) = t;
-  }
-  __syncthreads();
-}
+// What a kernel's per-thread sums are: <.,.> alone (in .a, .b of the partial),
+// with a squared norm in .c or in .d, or the norm alone in .c.
+enum { SUM_DOT = 0, SUM_DOT_C = 1, SUM_DOT_D = 2, SUM_NORM = 3 };
 
-// As block_reduce_store2 for each group of ST threads of a block of PPB * ST
-// threads; groups with store == false only take part in the barriers.
-template <int PPB>
-__device__ __forceinline__ void group_reduce_store2(D4S v0, D4S v1, D4S *dst0, D4S *dst1, bool store) {
-  __shared__ D4S sh[PPB][2][ST / 32];
+// Fixed-order block sums of the two members of a pair, for each group of ST
+// threads of a block of PPB * ST threads: FP32 per-thread terms, FP64 sums, one
+// partial per member stored by groups with store == true (every thread takes
+// part in the barriers).
+// The FP64 pipe is the scarce unit here: a warp-wide FP64 add occupies it for
+// about 70 cycles, so summing all eight fields of two D4S down a shuffle tree
+// (40 adds a warp, and 8 conversions) took longer than the loads of the kernels
+// that end with it.  At each step a lane hands over the half of its values that
+// its partner keeps (members at distance 16, then norm / dot, then re / im), so
+// a warp does 8 FP64 adds (6 without a norm, 5 for the norm alone), and the
+// terms are widened by integer operations (exact).
+// 16^3 x 32, 384 right-hand sides: k_pair_xr 2.15 -> 1.68 ms (10.9 GB: 0.96 of the
+// measured copy rate), k_pair_copy 1.30 -> 0.94 ms, k_hop_pair with the TS epilogue
+// 2.02 -> 1.77 ms and with DOTR 1.99 -> 1.88 ms (variant 1, 8 blocks per SM).
+template <int PPB, int SUM>
+__device__ __forceinline__ void pair_reduce_store(float2 re, float2 im, float2 nn, D4S *dst0, D4S *dst1, bool store) {
+  __shared__ double sh[PPB][ST / 32][2][3];
   const int grp = threadIdx.x / ST, tid = threadIdx.x % ST;
   const int lane = tid & 31, w = tid >> 5;
-  v0.a = warp_sum_d(v0.a);
-  v0.b = warp_sum_d(v0.b);
-  v0.c = warp_sum_d(v0.c);
-  v0.d = warp_sum_d(v0.d);
-  v1.a = warp_sum_d(v1.a);
-  v1.b = warp_sum_d(v1.b);
-  v1.c = warp_sum_d(v1.c);
-  v1.d = warp_sum_d(v1.d);
-  if (lane == 0) {
-    sh[grp][0][w] = v0;
-    sh[grp][1][w] = v1;
+  const bool m1 = lane & 16, up8 = lane & 8, up4 = lane & 4;
+  constexpr bool DOT = SUM != SUM_NORM, NORM = SUM != SUM_DOT;
+  auto swap_members = [&](float2 f) {  // own member's term here + the partner lane's
+    const float other = __shfl_xor_sync(0xffffffffu, m1 ? f.x : f.y, 16);
+    return f32_to_f64_bits(m1 ? f.y : f.x) + f32_to_f64_bits(other);
+  };
+  auto add_xor = [&](double v, int o) { return v + __shfl_xor_sync(0xffffffffu, v, o); };
+  double v = 0.0;
+  if constexpr (DOT && NORM) {
+    double r = swap_members(re), i = swap_members(im), q = swap_members(nn);
+    const double t = __shfl_xor_sync(0xffffffffu, up8 ? r : q, 8);
+    const double u = __shfl_xor_sync(0xffffffffu, i, 8);
+    const double rq = (up8 ? q : r) + t;  // lanes with bit 8 keep the norm, the others re and im
+    const double iq = up8 ? rq : i + u;
+    v = (up4 ? iq : rq) + __shfl_xor_sync(0xffffffffu, up4 ? rq : iq, 4);
+  } else if constexpr (DOT) {
+    const double r = swap_members(re), i = swap_members(im);
+    v = (up4 ? i : r) + __shfl_xor_sync(0xffffffffu, up4 ? r : i, 4);
+    v = add_xor(v, 8);
+  } else {
+    v = add_xor(add_xor(swap_members(nn), 8), 4);
   }
+  v = add_xor(add_xor(v, 2), 1);
+  if ((lane & 3) == 0) sh[grp][w][m1][NORM && (up8 || !DOT) ? 2 : (up4 ? 1 : 0)] = v;
   __syncthreads();
-  if (tid < 2 && store) {
-    D4S t = sh[grp][tid][0];
+  if (tid < 8 && store) {
+    const int m = tid >> 2, f = tid & 3;  // member, field of the partial
+    const int kind = f < 2 ? (DOT ? f : -1) : (NORM && f == (SUM == SUM_DOT_D ? 3 : 2) ? 2 : -1);
+    double t = 0.0;
+    if (kind >= 0) {
+      t = sh[grp][0][m][kind];
 #pragma unroll
-    for (int k = 1; k < ST / 32; ++k) {
-      t.a += sh[grp][tid][k].a;
-      t.b += sh[grp][tid][k].b;
-      t.c += sh[grp][tid][k].c;
-      t.d += sh[grp][tid][k].d;
+      for (int k = 1; k < ST / 32; ++k) t += sh[grp][k][m][kind];
     }
-    *(tid ? dst1 : dst0) = t;
+    reinterpret_cast<double *>(m ? dst1 : dst0)[f] = t;
   }
   __syncthreads();
 }
@@ -352,7 +349,7 @@ __global__ void __launch_bounds__(ST, 4) k_hop32x2(Geom g, int p_out, const floa
     const bool two = j + 1 < cnt;
     const int rhs[2] = {list[j], two ? list[j + 1] : list[j]};
     const int i = sb * ST + threadIdx.x;
-    D4S red[2] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+    float2 red = make_float2(0.f, 0.f);  // |out|^2 of the two right-hand sides
     if (i < g.Vh) {
       int c[4];
       coords_of(g, p_out, i, c);
@@ -389,12 +386,13 @@ __global__ void __launch_bounds__(ST, 4) k_hop32x2(Geom g, int p_out, const floa
           float nn = 0.f;
 #pragma unroll
           for (int k = 0; k < 12; ++k) nn += o[k].x * o[k].x + o[k].y * o[k].y;
-          red[r].c = nn;
+          (r == 0 ? red.x : red.y) = nn;
         }
       }
     }
-    if (EPI == EPI_RES)
-      block_reduce_store2(red[0], red[1], part + (size_t)rhs[0] * nbx + sb, part + (size_t)rhs[1] * nbx + sb);
+    if (EPI == EPI_RES)  // an odd last entry has only one right-hand side (its second sum is not stored)
+      pair_reduce_store<1, SUM_NORM>(red, red, red, part + (size_t)rhs[0] * nbx + sb,
+                                     part + (size_t)rhs[1] * nbx + sb, true);
   }
 }
 
@@ -573,12 +571,11 @@ __device__ __forceinline__ void hop_dir_pair(const Geom &g, int p_out, const int
 }
 
 // Epilogue of the pair hopping term at output site i of pair P: o = cH acc
-// (+ cA a unless EPI_PLAIN), stored to out; EPI_DOTR: partials <B, o> per
-// member; EPI_TS: partials <o, a> and |o|^2 per member (r0, r1 untouched for
-// EPI_PLAIN).
+// (+ cA a unless EPI_PLAIN), stored to out; EPI_DOTR: this site's terms of <B, o> per
+// member; EPI_TS: terms of <o, a> and |o|^2 per member (untouched for EPI_PLAIN).
 template <class SP, int EPI>
 __device__ __forceinline__ void pair_epilogue(const CP acc[4][3], const float2 a[24], float2 cA2, float2 cH2,
-                                              const SP &out, const SP &B, int P, int i, D4S &r0, D4S &r1) {
+                                              const SP &out, const SP &B, int P, int i, float2 &sre, float2 &sim, float2 &snn) {
   float2 o[24];
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
@@ -601,9 +598,8 @@ __device__ __forceinline__ void pair_epilogue(const CP acc[4][3], const float2 a
       ip = F2(rb[2 * k], o[2 * k + 1], ip);
       im = F2(rb[2 * k + 1], o[2 * k], im);
     }
-    const float2 imag = S2(ip, im);
-    r0 = D4S{re.x, imag.x, 0, 0};
-    r1 = D4S{re.y, imag.y, 0, 0};
+    sre = re;
+    sim = S2(ip, im);
   } else if (EPI == EPI_TS) {  // <out, A> and |out|^2
     float2 re = make_float2(0.f, 0.f), ip = re, im = re, nn = re;
 #pragma unroll
@@ -615,9 +611,9 @@ __device__ __forceinline__ void pair_epilogue(const CP acc[4][3], const float2 a
       nn = F2(o[2 * k], o[2 * k], nn);
       nn = F2(o[2 * k + 1], o[2 * k + 1], nn);
     }
-    const float2 imag = S2(ip, im);
-    r0 = D4S{re.x, imag.x, 0, nn.x};
-    r1 = D4S{re.y, imag.y, 0, nn.y};
+    sre = re;
+    sim = S2(ip, im);
+    snn = nn;
   }
 }
 
@@ -643,7 +639,7 @@ __global__ void __launch_bounds__(ST * PPB, MINB) k_hop_pair(Geom g, int p_out, 
     const int i = sb * ST + tid;
     if (prof && tid == 0 && valid)
       atomicAdd(prof + EPI, (unsigned long long)min(ST, g.Vh - sb * ST) * (2 * P + 1 < nrhs ? 2 : 1));
-    D4S r0 = {0, 0, 0, 0}, r1 = {0, 0, 0, 0};
+    float2 sre = make_float2(0.f, 0.f), sim = sre, snn = sre;
     if (valid && i < g.Vh) {
       int c[4];
       coords_of(g, p_out, i, c);
@@ -658,11 +654,11 @@ __global__ void __launch_bounds__(ST * PPB, MINB) k_hop_pair(Geom g, int p_out, 
       hop_dir_pair<3, SP, R12>(g, p_out, c, i, in, P, links, acc);
       float2 a[24];
       if (EPI != EPI_PLAIN) load_scaled(A, P, i, a);
-      pair_epilogue<SP, EPI>(acc, a, cA2, cH2, out, B, P, i, r0, r1);
+      pair_epilogue<SP, EPI>(acc, a, cA2, cH2, out, B, P, i, sre, sim, snn);
     }
     if (EPI == EPI_DOTR || EPI == EPI_TS)
-      group_reduce_store2<PPB>(r0, r1, part + (size_t)(2 * P) * nbx + sb, part + (size_t)(2 * P + 1) * nbx + sb,
-                               valid);
+      pair_reduce_store<PPB, EPI == EPI_TS ? SUM_DOT_D : SUM_DOT>(
+          sre, sim, snn, part + (size_t)(2 * P) * nbx + sb, part + (size_t)(2 * P + 1) * nbx + sb, valid);
   }
 }
 
@@ -780,10 +776,11 @@ __global__ void __launch_bounds__(ST, 3) k_hop_pair_pl(Geom g, int p_out, const 
     hop_dir_plane<3>(g, p_out, c, i, pl_sm, links, acc);
     float2 a[24];
     if (EPI != EPI_PLAIN) load_plane(pl_sm, PL_SLOTS, tid, a);
-    D4S r0 = {0, 0, 0, 0}, r1 = {0, 0, 0, 0};
-    pair_epilogue<BF16P, EPI>(acc, a, cA2, cH2, out, B, P, i, r0, r1);
+    float2 sre = make_float2(0.f, 0.f), sim = sre, snn = sre;
+    pair_epilogue<BF16P, EPI>(acc, a, cA2, cH2, out, B, P, i, sre, sim, snn);
     if (EPI == EPI_DOTR || EPI == EPI_TS)
-      group_reduce_store2<1>(r0, r1, part + (size_t)(2 * P) * nbx + sb, part + (size_t)(2 * P + 1) * nbx + sb, true);
+      pair_reduce_store<1, EPI == EPI_TS ? SUM_DOT_D : SUM_DOT>(
+          sre, sim, snn, part + (size_t)(2 * P) * nbx + sb, part + (size_t)(2 * P + 1) * nbx + sb, true);
     __syncthreads();  // the next item's copies overwrite the planes
   }
 }
@@ -1228,7 +1225,7 @@ __global__ void __launch_bounds__(ST) k_pair_xr(int vh, const SState *sc, const 
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     const int P = plist[w / nbx], sb = w % nbx;
     const int i = sb * ST + threadIdx.x;
-    D4S r0 = {0, 0, 0, 0}, r1 = {0, 0, 0, 0};
+    float2 sre = make_float2(0.f, 0.f), sim = sre, snn = sre;
     if (i < vh) {
       const bool a0 = flags[2 * P] & FLAG_ACTIVE, a1 = flags[2 * P + 1] & FLAG_ACTIVE;
       const CP al = scal_pair(sc[2 * P].alpha, sc[2 * P + 1].alpha);
@@ -1265,11 +1262,12 @@ __global__ void __launch_bounds__(ST) k_pair_xr(int vh, const SState *sc, const 
         nn = F2(sv[2 * k], sv[2 * k], nn);
         nn = F2(sv[2 * k + 1], sv[2 * k + 1], nn);
       }
-      const float2 imag = S2(ip, im);
-      r0 = D4S{re.x, imag.x, nn.x, 0};
-      r1 = D4S{re.y, imag.y, nn.y, 0};
+      sre = re;
+      sim = S2(ip, im);
+      snn = nn;
     }
-    block_reduce_store2(r0, r1, part + (size_t)(2 * P) * nbx + sb, part + (size_t)(2 * P + 1) * nbx + sb);
+    pair_reduce_store<1, SUM_DOT_C>(sre, sim, snn, part + (size_t)(2 * P) * nbx + sb,
+                                    part + (size_t)(2 * P + 1) * nbx + sb, true);
   }
 }
 
@@ -1283,7 +1281,7 @@ __global__ void __launch_bounds__(ST) k_pair_copy(int vh, const int *flags, F32F
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     const int P = plist[w / nbx], sb = w % nbx;
     const int i = sb * ST + threadIdx.x;
-    D4S r0 = {0, 0, 0, 0}, r1 = {0, 0, 0, 0};
+    float2 sre = make_float2(0.f, 0.f), sim = sre, snn = sre;
     if (i < vh) {
       const bool w0 = flags[2 * P] & FLAG_RU, w1 = flags[2 * P + 1] & FLAG_RU;
       float2 s0[12], s1[12], v[24];
@@ -1315,11 +1313,12 @@ __global__ void __launch_bounds__(ST) k_pair_copy(int vh, const int *flags, F32F
         nn = F2(v[2 * k], v[2 * k], nn);
         nn = F2(v[2 * k + 1], v[2 * k + 1], nn);
       }
-      const float2 imag = S2(ip, im);
-      r0 = D4S{re.x, imag.x, nn.x, 0};
-      r1 = D4S{re.y, imag.y, nn.y, 0};
+      sre = re;
+      sim = S2(ip, im);
+      snn = nn;
     }
-    block_reduce_store2(r0, r1, part + (size_t)(2 * P) * nbx + sb, part + (size_t)(2 * P + 1) * nbx + sb);
+    pair_reduce_store<1, SUM_DOT_C>(sre, sim, snn, part + (size_t)(2 * P) * nbx + sb,
+                                    part + (size_t)(2 * P + 1) * nbx + sb, true);
   }
 }
 
