@@ -97,7 +97,7 @@ __global__ void k_pack_gauge(const double2 *__restrict__ U, Geom g, float4 *U32,
   for (int a = 0; a < 3; ++a)
     for (int b = 0; b < 3; ++b) {
       double2 acc = make_double2(0.0, 0.0);
-      for (int k = 0; k < 3; ++k) acc = cadd(acc, cmulc(m[k][a], m[k][b]));
+      for (int k = 0; k < 3; ++k) acc = cmacc(acc, m[k][a], m[k][b]);
       acc.x -= (a == b) ? 1.0 : 0.0;
       dev = fmax(dev, fmax(fabs(acc.x), fabs(acc.y)));
     }

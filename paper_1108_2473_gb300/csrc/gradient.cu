@@ -61,7 +61,7 @@ __global__ void k_adj_source(Geom g, const double2 *__restrict__ src, const doub
 #pragma unroll
       for (int col = 0; col < 3; ++col) {
         double2 gv = gphase(g_ph(gi, a), v[g_col(gi, a) * 3 + col]);
-        o[a * 3 + col] = cadd(o[a * 3 + col], cmul(c, gv));
+        o[a * 3 + col] = cmac(o[a * 3 + col], c, gv);
       }
   }
   double2 *out = eta + idx * 12;
@@ -100,14 +100,15 @@ __device__ __forceinline__ void half_proj(const double2 *__restrict__ v, double2
   }
 }
 
-// out_ij += sum_{a=0,1} conj(a_ai) b_aj
+// out_ij += sum_{a=0,1} conj(a_ai) b_aj (FP64-pipe bound: chains of fused
+// multiply-adds, 144 operations instead of 216 per direction and right-hand side)
 __device__ __forceinline__ void outer_acc2(const double2 a[6], const double2 b[6], double2 out[3][3]) {
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) out[i][j] = cadd(out[i][j], cmulc(a[sp * 3 + i], b[sp * 3 + j]));
+      for (int j = 0; j < 3; ++j) out[i][j] = cmacc(out[i][j], a[sp * 3 + i], b[sp * 3 + j]);
 }
 
 // Link (s, MU): X = sum_r chi_r(x)^+ (1 - gamma_mu) phi_r(x+mu) and
