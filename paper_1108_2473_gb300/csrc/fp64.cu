@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "fx64.cuh"
 
 namespace lqcd {
 
@@ -100,22 +101,215 @@ __global__ void __launch_bounds__(128) k_hop64(Geom g, int p_out, const double2 
   }
 }
 
+// The same with the SU(3) products on the integer units (fx64.cuh), for SU(3) links.
+// Two threads per site: thread hs holds the projected row hs of every neighbour
+// (spin row hs and the lower row it is paired with), so that neither repeats a
+// conversion, and accumulates its upper output row and its shares of the two lower
+// ones; the shares that belong to the other thread change hands by one shuffle at the
+// end.  The eight directions are two loop bodies (real and imaginary spin phase):
+// unrolled eight times the code does not fit the instruction cache, and 42% of the
+// stalls were instruction fetches (2.79 ms for D on 12 right-hand sides of 16^3 x 32,
+// against 2.63 ms for FP64 arithmetic and 1.31 ms now).
+// Bound by instruction issue: per direction and right-hand side 108 integer
+// multiply-adds (2 cycles each), 12 conversions to integers of about 14 instructions,
+// and about as much again for the splits, the alignment and the sums.
+constexpr int HOP_SH = 4;  // eight directions of |X| < 2.45 * 2 * 2^57 stay below 2^63
+
+// direction mu = 2 J + (IMAG ? 0 : 1), runtime fwd; the spin phase of row hs is
+//   SG i (x), -+SG (y), +-SG i (z), SG (t) for hs = 0, 1
+template <bool DAG, bool IN_CANON, bool IMAG>
+__device__ __forceinline__ void hop_dir_fx(const Geom &g, int mu, bool fwd, int cm, int stride, int s, int hs,
+                                           const double2 *__restrict__ in, const int4 *__restrict__ U,
+                                           long long up[6], long long lo[6], long long l01[6], int &Ea, bool &bad) {
+  const int L = g.L[mu];
+  const bool edge_site = fwd ? cm + 1 == L : cm == 0;
+  const int step = edge_site ? stride * (1 - L) : stride;
+  const int sn = fwd ? s + step : s - step;
+  int4 u[9];
+  fx_load_link(U + ((size_t)(fwd ? s : sn) * 4 + mu) * 9, !fwd, u);
+  const int MINUS = (int)0x80000000;
+  const int edge = (mu == 3 && edge_site) ? MINUS : 0;  // time boundary
+  const int cj = fwd ? 0 : MINUS;
+  const bool minus = ((mu == 1 && hs == 0) || (mu == 2 && hs == 1)) != (fwd != DAG);
+  const int sg = minus ? MINUS : 0;
+  const int low = mu < 2 ? 3 - hs : 2 + hs;
+  const double2 *p = in + (size_t)(IN_CANON ? sn : (sn >> 1)) * 12;
+  double2 pu[3], pl[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    pu[k] = p[hs * 3 + k];
+    pl[k] = p[low * 3 + k];
+  }
+  int m = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) m = fx_max(fx_max(m, pu[k]), pl[k]);
+  const int E = m >> 20;
+  if (E < FX_EMIN || E > FX_EMAX) {  // zero contributes nothing; otherwise FP64
+    unsigned any = 0u;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      any |= __double2loint(pu[k].x) | __double2loint(pu[k].y) | __double2loint(pl[k].x) | __double2loint(pl[k].y);
+    bad = bad || m != 0 || any != 0u;
+    return;
+  }
+  long long h[6], X[6];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const long long ur = fx_int<HOP_SH>(pu[k].x, E, edge), ui = fx_int<HOP_SH>(pu[k].y, E, edge ^ cj);
+    if (IMAG) {  // + SG i l
+      h[2 * k] = ur - fx_int<HOP_SH>(pl[k].y, E, edge ^ sg);
+      h[2 * k + 1] = ui + fx_int<HOP_SH>(pl[k].x, E, edge ^ sg ^ cj);
+    } else {  // + SG l
+      h[2 * k] = ur + fx_int<HOP_SH>(pl[k].x, E, edge ^ sg);
+      h[2 * k + 1] = ui + fx_int<HOP_SH>(pl[k].y, E, edge ^ sg ^ cj);
+    }
+  }
+  fx_su3(u, h, X);
+  if (E > Ea) {
+    const int d = min(E - Ea, 63);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      up[k] >>= d;
+      lo[k] >>= d;
+      l01[k] >>= d;
+    }
+    Ea = E;
+  }
+  const int d = min(Ea - E, 63);
+  const long long ncj = cj >> 31, nsg = sg >> 31;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const long long xr = X[2 * k] >> d, xi = fx_negif(X[2 * k + 1] >> d, ncj);
+    up[2 * k] += xr;
+    up[2 * k + 1] += xi;
+    if (IMAG) {  // the conjugate phase: - SG i x
+      lo[2 * k] += fx_negif(xi, nsg);
+      lo[2 * k + 1] -= fx_negif(xr, nsg);
+    } else {  // + SG x
+      lo[2 * k] += fx_negif(xr, nsg);
+      lo[2 * k + 1] += fx_negif(xi, nsg);
+    }
+  }
+}
+
+// H in at one site in FP64: rows hs and 2 + hs
+template <bool DAG, bool IN_CANON>
+__device__ __noinline__ void hop_site64(const Geom &g, int p_out, int i, int hs, const double2 *in, const double2 *U,
+                                        double2 out[6]) {
+  int c[4];
+  coords_of(g, p_out, i, c);
+  const int s = site_of(g, c);
+  double2 acc[4][3];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) acc[a][b] = make_double2(0.0, 0.0);
+  hop_dir64<0, DAG, IN_CANON>(g, c, s, in, U, acc);
+  hop_dir64<1, DAG, IN_CANON>(g, c, s, in, U, acc);
+  hop_dir64<2, DAG, IN_CANON>(g, c, s, in, U, acc);
+  hop_dir64<3, DAG, IN_CANON>(g, c, s, in, U, acc);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    out[k] = hs ? acc[1][k] : acc[0][k];
+    out[3 + k] = hs ? acc[3][k] : acc[2][k];
+  }
+}
+
+template <bool DAG, bool IN_CANON, bool OUT_CANON>
+__global__ void __launch_bounds__(128, 3) k_hop64_fx(Geom g, int p_out, const double2 *__restrict__ U,
+                                                  const int4 *__restrict__ Ufx, const double2 *__restrict__ in,
+                                                  size_t in_stride, double2 *out, size_t out_stride, const double2 *A,
+                                                  double cA, const double2 *B, double cB, double cH,
+                                                  const int *active) {
+  const int rhs = blockIdx.y;
+  if (active && !active[rhs]) return;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = min(idx >> 1, g.Vh - 1), hs = idx & 1;  // past the end: repeats the last site, stores nothing
+  int c[4];
+  coords_of(g, p_out, i, c);
+  const int s = site_of(g, c);
+  const double2 *inr = in + (size_t)rhs * in_stride;
+  long long up[6], lo[6], l01[6];
+  int Ea = FX_EMIN;
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) up[k] = lo[k] = l01[k] = 0;
+  const int s2 = g.L[0] * g.L[1], s3 = s2 * g.L[2];
+#pragma unroll 1
+  for (int j = 0; j < 2; ++j) {
+    if (j == 1) {  // lo holds the shares of mu = x, y from here on in l01
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        l01[k] = lo[k];
+        lo[k] = 0;
+      }
+    }
+#pragma unroll 1
+    for (int f = 0; f < 2; ++f) {
+      hop_dir_fx<DAG, IN_CANON, true>(g, 2 * j, f == 0, j ? c[2] : c[0], j ? s2 : 1, s, hs, inr, Ufx, up, lo, l01, Ea,
+                                      bad);
+      hop_dir_fx<DAG, IN_CANON, false>(g, 2 * j + 1, f == 0, j ? c[3] : c[1], j ? s3 : g.L[0], s, hs, inr, Ufx, up, lo,
+                                       l01, Ea, bad);
+    }
+  }
+  // lower row 2 + hs: own shares of mu = z, t and the other thread's of x, y
+  const int Eo = __shfl_xor_sync(0xffffffffu, Ea, 1);
+  bad = bad || __shfl_xor_sync(0xffffffffu, (int)bad, 1);
+  long long ot[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) ot[k] = __shfl_xor_sync(0xffffffffu, l01[k], 1);
+  if ((idx >> 1) >= g.Vh) return;
+  double2 v[6];
+  if (bad) {
+    hop_site64<DAG, IN_CANON>(g, p_out, i, hs, inr, U, v);
+  } else {
+    int El = Ea;
+    const int dl = fx_align<6>(lo, El, Eo);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      v[k] = make_double2(fx_double<HOP_SH>(up[2 * k], Ea), fx_double<HOP_SH>(up[2 * k + 1], Ea));
+      v[3 + k] = make_double2(fx_double<HOP_SH>(lo[2 * k] + (ot[2 * k] >> dl), El),
+                              fx_double<HOP_SH>(lo[2 * k + 1] + (ot[2 * k + 1] >> dl), El));
+    }
+  }
+  const size_t o = (size_t)rhs * out_stride + (size_t)(OUT_CANON ? s : i) * 12 + hs * 3;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const size_t e = o + (k < 3 ? k : 3 + k);  // rows hs and 2 + hs
+    double2 w = v[k];
+    if (A) {  // one fused multiply-add per component where cA = 1, the usual call
+      const double2 a = A[e], t = cA == 1.0 ? a : cscale(a, cA);
+      w = make_double2(fma(cH, w.x, t.x), fma(cH, w.y, t.y));
+    } else if (cH != 1.0) {
+      w = cscale(w, cH);
+    }
+    if (B) {
+      const double2 b = B[e];
+      w = make_double2(fma(cB, b.x, w.x), fma(cB, b.y, w.y));
+    }
+    out[e] = w;
+  }
+}
+
 int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
                  const double2 *in, size_t in_stride, double2 *out, size_t out_stride, const double2 *A, double cA,
                  const double2 *B, double cB, double cH, const int *active, int nrhs) {
   const Geom &g = ctx->geom;
-  dim3 grid((g.Vh + 127) / 128, nrhs);
-#define HOP64_CASE(D, IC, OC)                                                                          \
-  if (dag == D && in_canon == IC && out_canon == OC) {                                                 \
-    KL k_hop64<D, IC, OC><<<grid, 128, 0, st>>>(g, p_out, ctx->U64, in, in_stride, out, out_stride, A, cA, B, cB, \
-                                             cH, active);                                              \
-    LQCD_LAUNCH_CHECK(ctx, "k_hop64");                                                                 \
-    return LQCD_OK;                                                                                    \
+  // links that are not SU(3) may be of any size: FP64 arithmetic
+  const dim3 grid((g.Vh + 127) / 128, nrhs), grid_fx((2 * (size_t)g.Vh + 127) / 128, nrhs);
+#define HOP64_CASE(D, IC, OC)                                                                                   \
+  if (dag == D && in_canon == IC && out_canon == OC) {                                                          \
+    if (!ctx->gauge_su3)                                                                                        \
+      KL k_hop64<D, IC, OC><<<grid, 128, 0, st>>>(g, p_out, ctx->U64, in, in_stride, out, out_stride, A, cA, B, \
+                                                  cB, cH, active);                                              \
+    else                                                                                                        \
+      KL k_hop64_fx<D, IC, OC><<<grid_fx, 128, 0, st>>>(g, p_out, ctx->U64, ctx->Ufx, in, in_stride, out,       \
+                                                        out_stride, A, cA, B, cB, cH, active);                  \
+    LQCD_LAUNCH_CHECK(ctx, "k_hop64");                                                                          \
+    return LQCD_OK;                                                                                             \
   }
   HOP64_CASE(false, false, false)
   HOP64_CASE(false, true, true)
-  HOP64_CASE(false, true, false)
-  HOP64_CASE(false, false, true)
   HOP64_CASE(true, true, true)
   HOP64_CASE(true, false, false)
 #undef HOP64_CASE
