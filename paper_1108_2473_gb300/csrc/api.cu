@@ -5,7 +5,7 @@
 #include <cmath>
 
 #include "internal.cuh"
-#include "fx64.cuh"
+#include "fxfield.cuh"
 
 using namespace lqcd;
 
@@ -76,8 +76,8 @@ __device__ __forceinline__ float to_tf32(float x) {
 
 // Check unitarity and unit determinant of every link; write the reduced-precision
 // copies (FP32 reconstruct-12, FP16 with all 18 reals duplicated, tf32,
-// double-float, integer limbs) in parity-split order.
-__global__ void k_pack_gauge(const double2 *__restrict__ U, Geom g, float4 *U32, uint4 *U16, float4 *Udf,
+// integer limbs) in parity-split order.
+__global__ void k_pack_gauge(const double2 *__restrict__ U, Geom g, float4 *U32, uint4 *U16,
                              float2 *Utf, int4 *Ufx, int *flag) {
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= g.V * 4) return;
@@ -87,14 +87,7 @@ __global__ void k_pack_gauge(const double2 *__restrict__ U, Geom g, float4 *U32,
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      m[a][b] = u[a * 3 + b];
-      // double-float copy for the residual: hi = fl32(v), lo = fl32(v - hi)
-      float hx = (float)m[a][b].x, hy = (float)m[a][b].y;
-      Udf[(size_t)idx * 9 + a * 3 + b] =
-          make_float4(hx, hy, (float)(m[a][b].x - (double)hx), (float)(m[a][b].y - (double)hy));
-      Ufx[(size_t)idx * 9 + a * 3 + b] = fx_link_entry(m[a][b].x, m[a][b].y);
-    }
+    for (int b = 0; b < 3; ++b) m[a][b] = u[a * 3 + b];
   double dev = 0.0;
   for (int a = 0; a < 3; ++a)
     for (int b = 0; b < 3; ++b) {
@@ -114,6 +107,11 @@ __global__ void k_pack_gauge(const double2 *__restrict__ U, Geom g, float4 *U32,
   int p = (x + y + z + t) & 1;
   int i = s >> 1;
   size_t base = ((size_t)(p * 4 + mu) * 3) * g.Vh + i;
+  // integer limbs with the sign of the time boundary (hops over t = Lt - 1 <-> 0)
+  const double tsgn = (mu == 3 && t == g.L[3] - 1) ? -1.0 : 1.0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k)
+    Ufx[fx_link_index(p, mu, g.Vh, i) + 32 * k] = fx_link_entry(tsgn * m[k / 3][k % 3].x, tsgn * m[k / 3][k % 3].y);
   float v[12];
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
@@ -251,9 +249,9 @@ int lqcd_destroy(lqcd_ctx *ctx) {
   cudaFree(ctx->Utf);
   cudaFree(ctx->Ub16);
   cudaFree(ctx->Uape);
-  cudaFree(ctx->Udf);
   cudaFree(ctx->Ufx);
   cudaFree(ctx->Uapefx);
+  if (ctx->fx_ev) cudaEventDestroy(ctx->fx_ev);
   cudaFree(ctx->d_flag);
   cudaFree(ctx->d_prof);
   for (cudaEvent_t e : ctx->prof_ev) cudaEventDestroy(e);
@@ -286,8 +284,7 @@ static int set_gauge_impl(lqcd_ctx *ctx, const double *U, lqcd_stream_t stream, 
     LQCD_CUDA_TRY(ctx, cudaMalloc(&ctx->U32, (size_t)g.V * 4 * 3 * sizeof(float4)));
     LQCD_CUDA_TRY(ctx, cudaMalloc(&ctx->U16, (size_t)g.Vh * 2 * 4 * 5 * sizeof(uint4)));
     LQCD_CUDA_TRY(ctx, cudaMalloc(&ctx->Utf, (size_t)g.Vh * 2 * 4 * 9 * sizeof(float2)));
-    LQCD_CUDA_TRY(ctx, cudaMalloc(&ctx->Udf, n64 * sizeof(float4)));
-    LQCD_CUDA_TRY(ctx, cudaMalloc(&ctx->Ufx, n64 * sizeof(int4)));
+    LQCD_CUDA_TRY(ctx, cudaMalloc(&ctx->Ufx, (size_t)fx_blocks(g.Vh) * 8 * 288 * sizeof(int4)));
   }
   int st_ = LQCD_OK;
   double2 *stage = (double2 *)workspace(ctx, WS_STAGE_AUX, n64 * sizeof(double2), &st_);
@@ -296,7 +293,7 @@ static int set_gauge_impl(lqcd_ctx *ctx, const double *U, lqcd_stream_t stream, 
   LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(stage, U, n64 * sizeof(double2), kind, st));
   LQCD_CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), st));
   int threads = 256, blocks = (g.V * 4 + threads - 1) / threads;
-  KL k_pack_gauge<<<blocks, threads, 0, st>>>(stage, g, ctx->U32, ctx->U16, ctx->Udf, ctx->Utf, ctx->Ufx, ctx->d_flag);
+  KL k_pack_gauge<<<blocks, threads, 0, st>>>(stage, g, ctx->U32, ctx->U16, ctx->Utf, ctx->Ufx, ctx->d_flag);
   LQCD_LAUNCH_CHECK(ctx, "k_pack_gauge");
   int flag = 0;
   LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(&flag, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -5,11 +5,12 @@
 // Layouts: canonical fields are [rhs][V][12] double2 (site-lexicographic);
 // solver vectors are parity-compact [rhs][Vh][12] double2 with parity-local
 // index i = site >> 1.  The gauge field is the canonical [V][4][9] copy.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
 #include "internal.cuh"
-#include "fx64.cuh"
+#include "fxfield.cuh"
 
 namespace lqcd {
 
@@ -101,97 +102,6 @@ __global__ void __launch_bounds__(128) k_hop64(Geom g, int p_out, const double2 
   }
 }
 
-// The same with the SU(3) products on the integer units (fx64.cuh), for SU(3) links.
-// Two threads per site: thread hs holds the projected row hs of every neighbour
-// (spin row hs and the lower row it is paired with), so that neither repeats a
-// conversion, and accumulates its upper output row and its shares of the two lower
-// ones; the shares that belong to the other thread change hands by one shuffle at the
-// end.  The eight directions are two loop bodies (real and imaginary spin phase):
-// unrolled eight times the code does not fit the instruction cache, and 42% of the
-// stalls were instruction fetches (2.79 ms for D on 12 right-hand sides of 16^3 x 32,
-// against 2.63 ms for FP64 arithmetic and 1.31 ms now).
-// Bound by instruction issue: per direction and right-hand side 108 integer
-// multiply-adds (2 cycles each), 12 conversions to integers of about 14 instructions,
-// and about as much again for the splits, the alignment and the sums.
-constexpr int HOP_SH = 4;  // eight directions of |X| < 2.45 * 2 * 2^57 stay below 2^63
-
-// direction mu = 2 J + (IMAG ? 0 : 1), runtime fwd; the spin phase of row hs is
-//   SG i (x), -+SG (y), +-SG i (z), SG (t) for hs = 0, 1
-template <bool DAG, bool IN_CANON, bool IMAG>
-__device__ __forceinline__ void hop_dir_fx(const Geom &g, int mu, bool fwd, int cm, int stride, int s, int hs,
-                                           const double2 *__restrict__ in, const int4 *__restrict__ U,
-                                           long long up[6], long long lo[6], long long l01[6], int &Ea, bool &bad) {
-  const int L = g.L[mu];
-  const bool edge_site = fwd ? cm + 1 == L : cm == 0;
-  const int step = edge_site ? stride * (1 - L) : stride;
-  const int sn = fwd ? s + step : s - step;
-  int4 u[9];
-  fx_load_link(U + ((size_t)(fwd ? s : sn) * 4 + mu) * 9, !fwd, u);
-  const int MINUS = (int)0x80000000;
-  const int edge = (mu == 3 && edge_site) ? MINUS : 0;  // time boundary
-  const int cj = fwd ? 0 : MINUS;
-  const bool minus = ((mu == 1 && hs == 0) || (mu == 2 && hs == 1)) != (fwd != DAG);
-  const int sg = minus ? MINUS : 0;
-  const int low = mu < 2 ? 3 - hs : 2 + hs;
-  const double2 *p = in + (size_t)(IN_CANON ? sn : (sn >> 1)) * 12;
-  double2 pu[3], pl[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    pu[k] = p[hs * 3 + k];
-    pl[k] = p[low * 3 + k];
-  }
-  int m = 0;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) m = fx_max(fx_max(m, pu[k]), pl[k]);
-  const int E = m >> 20;
-  if (E < FX_EMIN || E > FX_EMAX) {  // zero contributes nothing; otherwise FP64
-    unsigned any = 0u;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      any |= __double2loint(pu[k].x) | __double2loint(pu[k].y) | __double2loint(pl[k].x) | __double2loint(pl[k].y);
-    bad = bad || m != 0 || any != 0u;
-    return;
-  }
-  long long h[6], X[6];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const long long ur = fx_int<HOP_SH>(pu[k].x, E, edge), ui = fx_int<HOP_SH>(pu[k].y, E, edge ^ cj);
-    if (IMAG) {  // + SG i l
-      h[2 * k] = ur - fx_int<HOP_SH>(pl[k].y, E, edge ^ sg);
-      h[2 * k + 1] = ui + fx_int<HOP_SH>(pl[k].x, E, edge ^ sg ^ cj);
-    } else {  // + SG l
-      h[2 * k] = ur + fx_int<HOP_SH>(pl[k].x, E, edge ^ sg);
-      h[2 * k + 1] = ui + fx_int<HOP_SH>(pl[k].y, E, edge ^ sg ^ cj);
-    }
-  }
-  fx_su3(u, h, X);
-  if (E > Ea) {
-    const int d = min(E - Ea, 63);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      up[k] >>= d;
-      lo[k] >>= d;
-      l01[k] >>= d;
-    }
-    Ea = E;
-  }
-  const int d = min(Ea - E, 63);
-  const long long ncj = cj >> 31, nsg = sg >> 31;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const long long xr = X[2 * k] >> d, xi = fx_negif(X[2 * k + 1] >> d, ncj);
-    up[2 * k] += xr;
-    up[2 * k + 1] += xi;
-    if (IMAG) {  // the conjugate phase: - SG i x
-      lo[2 * k] += fx_negif(xi, nsg);
-      lo[2 * k + 1] -= fx_negif(xr, nsg);
-    } else {  // + SG x
-      lo[2 * k] += fx_negif(xr, nsg);
-      lo[2 * k + 1] += fx_negif(xi, nsg);
-    }
-  }
-}
-
 // H in at one site in FP64: rows hs and 2 + hs
 template <bool DAG, bool IN_CANON>
 __device__ __noinline__ void hop_site64(const Geom &g, int p_out, int i, int hs, const double2 *in, const double2 *U,
@@ -215,67 +125,12 @@ __device__ __noinline__ void hop_site64(const Geom &g, int p_out, int i, int hs,
   }
 }
 
-template <bool DAG, bool IN_CANON, bool OUT_CANON>
-__global__ void __launch_bounds__(128, 3) k_hop64_fx(Geom g, int p_out, const double2 *__restrict__ U,
-                                                  const int4 *__restrict__ Ufx, const double2 *__restrict__ in,
-                                                  size_t in_stride, double2 *out, size_t out_stride, const double2 *A,
-                                                  double cA, const double2 *B, double cB, double cH,
-                                                  const int *active) {
-  const int rhs = blockIdx.y;
-  if (active && !active[rhs]) return;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = min(idx >> 1, g.Vh - 1), hs = idx & 1;  // past the end: repeats the last site, stores nothing
-  int c[4];
-  coords_of(g, p_out, i, c);
-  const int s = site_of(g, c);
-  const double2 *inr = in + (size_t)rhs * in_stride;
-  long long up[6], lo[6], l01[6];
-  int Ea = FX_EMIN;
-  bool bad = false;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) up[k] = lo[k] = l01[k] = 0;
-  const int s2 = g.L[0] * g.L[1], s3 = s2 * g.L[2];
-#pragma unroll 1
-  for (int j = 0; j < 2; ++j) {
-    if (j == 1) {  // lo holds the shares of mu = x, y from here on in l01
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        l01[k] = lo[k];
-        lo[k] = 0;
-      }
-    }
-#pragma unroll 1
-    for (int f = 0; f < 2; ++f) {
-      hop_dir_fx<DAG, IN_CANON, true>(g, 2 * j, f == 0, j ? c[2] : c[0], j ? s2 : 1, s, hs, inr, Ufx, up, lo, l01, Ea,
-                                      bad);
-      hop_dir_fx<DAG, IN_CANON, false>(g, 2 * j + 1, f == 0, j ? c[3] : c[1], j ? s3 : g.L[0], s, hs, inr, Ufx, up, lo,
-                                       l01, Ea, bad);
-    }
-  }
-  // lower row 2 + hs: own shares of mu = z, t and the other thread's of x, y
-  const int Eo = __shfl_xor_sync(0xffffffffu, Ea, 1);
-  bad = bad || __shfl_xor_sync(0xffffffffu, (int)bad, 1);
-  long long ot[6];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) ot[k] = __shfl_xor_sync(0xffffffffu, l01[k], 1);
-  if ((idx >> 1) >= g.Vh) return;
-  double2 v[6];
-  if (bad) {
-    hop_site64<DAG, IN_CANON>(g, p_out, i, hs, inr, U, v);
-  } else {
-    int El = Ea;
-    const int dl = fx_align<6>(lo, El, Eo);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      v[k] = make_double2(fx_double<HOP_SH>(up[2 * k], Ea), fx_double<HOP_SH>(up[2 * k + 1], Ea));
-      v[3 + k] = make_double2(fx_double<HOP_SH>(lo[2 * k] + (ot[2 * k] >> dl), El),
-                              fx_double<HOP_SH>(lo[2 * k + 1] + (ot[2 * k + 1] >> dl), El));
-    }
-  }
-  const size_t o = (size_t)rhs * out_stride + (size_t)(OUT_CANON ? s : i) * 12 + hs * 3;
+// out = cA A + cB B + cH v at rows hs and 2 + hs (v) of one site, o: its row hs
+__device__ __forceinline__ void hop64_store(const double2 v[6], size_t o, double2 *out, const double2 *A, double cA,
+                                            const double2 *B, double cB, double cH) {
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    const size_t e = o + (k < 3 ? k : 3 + k);  // rows hs and 2 + hs
+    const size_t e = o + (k < 3 ? k : 3 + k);
     double2 w = v[k];
     if (A) {  // one fused multiply-add per component where cA = 1, the usual call
       const double2 a = A[e], t = cA == 1.0 ? a : cscale(a, cA);
@@ -291,20 +146,131 @@ __global__ void __launch_bounds__(128, 3) k_hop64_fx(Geom g, int p_out, const do
   }
 }
 
-int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
-                 const double2 *in, size_t in_stride, double2 *out, size_t out_stride, const double2 *A, double cA,
-                 const double2 *B, double cB, double cH, const int *active, int nrhs) {
+// FP64 field -> integer limbs: canonical (both parities) or the compact field of one
+// parity (f0).  Thread per site and right-hand side (grid.y).
+template <bool CANON>
+__global__ void __launch_bounds__(128) k_fx_from64(Geom g, const double2 *__restrict__ in, size_t in_stride, FxF f0,
+                                                   FxF f1, const int *active) {
+  const int rhs = blockIdx.y, idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (active && !active[rhs]) return;
+  if (idx >= (CANON ? g.V : g.Vh)) return;
+  int p = 0, i = idx;
+  if (CANON) {
+    int r = idx / g.L[0];
+    const int y = r % g.L[1];
+    r /= g.L[1];
+    p = (idx % g.L[0] + y + r % g.L[2] + r / g.L[2]) & 1;
+    i = idx >> 1;
+  }
+  const double2 *q = in + (size_t)rhs * in_stride + (size_t)idx * 12;
+  const FxF f = (p ? f1 : f0).at(rhs);
+  double2 v[12];
+  int m = 0;
+  unsigned low = 0u;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) v[k] = q[k];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    m = fx_max(m, v[k]);
+    low |= __double2loint(v[k].x) | __double2loint(v[k].y);
+  }
+  const int E = fx_site_exp(m, low);
+  f.e[i] = E;
+  if (E <= 0) return;  // the limbs of such a site are not read
+  int4 *o = f.site(i);
+#pragma unroll
+  for (int k = 0; k < 12; ++k)
+    o[32 * k] = fx_split_c(fx_int<FXF_SH>(v[k].x, E, 0), fx_int<FXF_SH>(v[k].y, E, 0));
+}
+
+// The hopping term with its SU(3) products on the integer units (fx64.cuh), on a field
+// of integer limbs (fxfield.cuh); the FP64 field `in` it was made from serves the sites
+// that have no integer form.  D on 12 right-hand sides of 16^3 x 32, conversion
+// included: 2.63 ms in FP64 arithmetic (k_hop64), 1.31 ms when each neighbour is
+// converted where it is used, 0.97 ms here; one right-hand side of 4^4: 28 us, as
+// in FP64.
+template <bool DAG, bool IN_CANON, bool OUT_CANON>
+__global__ void __launch_bounds__(128, 4) k_hop64_fxf(Geom g, int p_out, const double2 *__restrict__ U,
+                                                      const int4 *__restrict__ Ufx, FxF f,
+                                                      const double2 *__restrict__ in, size_t in_stride, double2 *out,
+                                                      size_t out_stride, const double2 *A, double cA, const double2 *B,
+                                                      double cB, double cH, const int *active) {
+  const int rhs = blockIdx.y, warp = threadIdx.x >> 5, hs = warp & 1;
+  if (active && !active[rhs]) return;
+  const int site = blockIdx.x * 64 + (warp >> 1) * 32 + (threadIdx.x & 31), i = min(site, g.Vh - 1);
+  long long up[6], low[6];
+  int Em;
+  bool bad;
+  fxf_hop<DAG>(g, p_out, i, hs, f.at(rhs), Ufx, up, low, Em, bad);
+  if (site >= g.Vh) return;
+  double2 v[6];
+  if (bad) {
+    hop_site64<DAG, IN_CANON>(g, p_out, i, hs, in + (size_t)rhs * in_stride, U, v);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      v[k] = make_double2(fx_double<FXF_SH>(up[2 * k], Em), fx_double<FXF_SH>(up[2 * k + 1], Em));
+      v[3 + k] = make_double2(fx_double<FXF_SH>(low[2 * k], Em), fx_double<FXF_SH>(low[2 * k + 1], Em));
+    }
+  }
+  size_t s = i;
+  if (OUT_CANON) {
+    int c[4];
+    coords_of(g, p_out, i, c);
+    s = site_of(g, c);
+  }
+  hop64_store(v, (size_t)rhs * out_stride + s * 12 + hs * 3, out, A, cA, B, cB, cH);
+}
+
+// Workspace of integer limbs for n_par parities of up to *chunk right-hand sides, or
+// null (then the caller takes FP64 arithmetic, as for links that are not SU(3), which
+// may be of any size): as many as keep it in L2 (FX_WS_BYTES), at least one.  Not while the stream is being captured, when nothing
+// may be allocated.  The workspace is shared by the context's streams: a call waits
+// for the last one's event, and fx_workspace_done records its own.
+constexpr size_t FX_WS_BYTES = 96u << 20;
+static char *fx_workspace(lqcd_ctx *ctx, int nrhs, int n_par, int *chunk, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  const size_t per = (size_t)n_par * fx_blocks(ctx->geom.Vh) * 32 * (12 * sizeof(int4) + sizeof(int));
+  *chunk = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FX_WS_BYTES / per));
+  int rc = LQCD_OK;
+  void *w = workspace(ctx, WS_FX, per * *chunk, &rc);
+  if (!w) return nullptr;
+  if (!ctx->fx_ev && cudaEventCreateWithFlags(&ctx->fx_ev, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    ctx->fx_ev = nullptr;
+    return nullptr;
+  }
+  if (ctx->fx_used && ctx->fx_stream != st && cudaStreamWaitEvent(st, ctx->fx_ev, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return (char *)w;
+}
+static int fx_workspace_done(lqcd_ctx *ctx, cudaStream_t st) {
+  LQCD_CUDA_TRY(ctx, cudaEventRecord(ctx->fx_ev, st));
+  ctx->fx_used = true;
+  ctx->fx_stream = st;
+  return LQCD_OK;
+}
+// one launch; fx: the input as integer limbs, or null
+static int launch_hop64_one(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
+                            const double2 *in, size_t in_stride, double2 *out, size_t out_stride, const double2 *A,
+                            double cA, const double2 *B, double cB, double cH, const int *active, int nrhs,
+                            const FxF *fx) {
   const Geom &g = ctx->geom;
-  // links that are not SU(3) may be of any size: FP64 arithmetic
-  const dim3 grid((g.Vh + 127) / 128, nrhs), grid_fx((2 * (size_t)g.Vh + 127) / 128, nrhs);
+  const dim3 grid((g.Vh + 127) / 128, nrhs);
 #define HOP64_CASE(D, IC, OC)                                                                                   \
   if (dag == D && in_canon == IC && out_canon == OC) {                                                          \
-    if (!ctx->gauge_su3)                                                                                        \
+    if (!fx)                                                                                                    \
       KL k_hop64<D, IC, OC><<<grid, 128, 0, st>>>(g, p_out, ctx->U64, in, in_stride, out, out_stride, A, cA, B, \
                                                   cB, cH, active);                                              \
     else                                                                                                        \
-      KL k_hop64_fx<D, IC, OC><<<grid_fx, 128, 0, st>>>(g, p_out, ctx->U64, ctx->Ufx, in, in_stride, out,       \
-                                                        out_stride, A, cA, B, cB, cH, active);                  \
+      KL k_hop64_fxf<D, IC, OC><<<dim3((g.Vh + 63) / 64, nrhs), 128, 0, st>>>(                                  \
+          g, p_out, ctx->U64, ctx->Ufx, *fx, in, in_stride, out, out_stride, A, cA, B, cB, cH, active);         \
     LQCD_LAUNCH_CHECK(ctx, "k_hop64");                                                                          \
     return LQCD_OK;                                                                                             \
   }
@@ -316,15 +282,67 @@ int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool o
   return set_error(ctx, LQCD_ERR_INVALID, "launch_hop64: unsupported layout combination");
 }
 
-int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, bool dagger, cudaStream_t st) {
+static FxF fx_carve(char *w, int p, int vh, int chunk) {
+  const int vb = fx_blocks(vh);
+  const size_t nd = (size_t)chunk * vb * 384;
+  return FxF{(int4 *)w + p * nd, (int *)((int4 *)w + 2 * nd) + (size_t)p * chunk * vb * 32, vb};
+}
+
+int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
+                 const double2 *in, size_t in_stride, double2 *out, size_t out_stride, const double2 *A, double cA,
+                 const double2 *B, double cB, double cH, const int *active, int nrhs) {
   const Geom &g = ctx->geom;
-  size_t stride = (size_t)g.V * 12;
-  for (int p = 0; p < 2; ++p) {
-    int rc = launch_hop64(ctx, st, dagger, true, true, p, in, stride, out, stride, in, 1.0, nullptr, 0.0,
-                          -ctx->kappa, nullptr, nrhs);
+  int chunk = 0;
+  char *w = nullptr;
+  // (sized for both parities: a canonical field is converted whole)
+  if (ctx->gauge_su3) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
+  if (!w)
+    return launch_hop64_one(ctx, st, dag, in_canon, out_canon, p_out, in, in_stride, out, out_stride, A, cA, B, cB, cH,
+                            active, nrhs, nullptr);
+  const FxF f0 = fx_carve(w, 0, g.Vh, chunk), f1 = fx_carve(w, 1, g.Vh, chunk);
+  for (int r = 0; r < nrhs; r += chunk) {
+    const int n = std::min(chunk, nrhs - r);
+    const int *act = active ? active + r : nullptr;
+    const double2 *inr = in + (size_t)r * in_stride;
+    const size_t o = (size_t)r * out_stride;
+    if (in_canon)
+      KL k_fx_from64<true><<<dim3((g.V + 127) / 128, n), 128, 0, st>>>(g, inr, in_stride, f0, f1, act);
+    else
+      KL k_fx_from64<false><<<dim3((g.Vh + 127) / 128, n), 128, 0, st>>>(g, inr, in_stride, f0, f0, act);
+    LQCD_LAUNCH_CHECK(ctx, "k_fx_from64");
+    const FxF &f = in_canon && p_out == 0 ? f1 : f0;  // the neighbours' parity
+    int rc = launch_hop64_one(ctx, st, dag, in_canon, out_canon, p_out, inr, in_stride, out + o, out_stride,
+                              A ? A + o : nullptr, cA, B ? B + o : nullptr, cB, cH, act, n, &f);
     if (rc) return rc;
   }
-  return LQCD_OK;
+  return fx_workspace_done(ctx, st);
+}
+
+int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, bool dagger, cudaStream_t st) {
+  const Geom &g = ctx->geom;
+  const size_t stride = (size_t)g.V * 12;
+  int chunk = nrhs;
+  char *w = nullptr;
+  if (ctx->gauge_su3) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
+  if (!w) chunk = nrhs;
+  for (int r = 0; r < nrhs; r += chunk) {
+    const int n = std::min(chunk, nrhs - r);
+    const double2 *inr = in + (size_t)r * stride;
+    double2 *outr = out + (size_t)r * stride;
+    FxF f[2];
+    if (w) {
+      f[0] = fx_carve(w, 0, g.Vh, chunk);
+      f[1] = fx_carve(w, 1, g.Vh, chunk);
+      KL k_fx_from64<true><<<dim3((g.V + 127) / 128, n), 128, 0, st>>>(g, inr, stride, f[0], f[1], nullptr);
+      LQCD_LAUNCH_CHECK(ctx, "k_fx_from64");
+    }
+    for (int p = 0; p < 2; ++p) {
+      int rc = launch_hop64_one(ctx, st, dagger, true, true, p, inr, stride, outr, stride, inr, 1.0, nullptr, 0.0,
+                                -ctx->kappa, nullptr, n, w ? &f[1 - p] : nullptr);
+      if (rc) return rc;
+    }
+  }
+  return w ? fx_workspace_done(ctx, st) : LQCD_OK;
 }
 
 // --------------------------------------------------------- layout changes

@@ -96,9 +96,9 @@ __device__ __forceinline__ void fx_su3(const int4 u[9], const long long h[6], lo
     X[2 * a + 1] = ai + ((bi + (1ll << 28)) >> 29);
   }
 }
-// the link, or its transpose
+// the link at w (entries 32 apart), or its transpose
 __device__ __forceinline__ void fx_load_link(const int4 *__restrict__ w, bool transpose, int4 u[9]) {
-  const int sa = transpose ? 1 : 3, sb = transpose ? 3 : 1;
+  const int sa = transpose ? 32 : 96, sb = transpose ? 96 : 32;
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll

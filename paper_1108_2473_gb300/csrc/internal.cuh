@@ -187,15 +187,17 @@ struct lqcd_ctx {
   bool gauge_su3 = false;     // links checked SU(3): reconstruct-12 copies are valid
   double2 *U64 = nullptr;     // canonical [V][4][3][3]
   float4 *U32 = nullptr;      // recon-12 FP32  [2 parity][4 mu][3 float4][Vh]
-  float4 *Udf = nullptr;      // double-float copy  [V][4][3][3] (hi.re, hi.im, lo.re, lo.im)
   uint4 *U16 = nullptr;       // FP16, all 18 reals, each twice  [2 parity][4 mu][5 uint4][Vh]
   float2 *Utf = nullptr;      // tf32-rounded FP32, [2 parity][4 mu][Vh][3][3] complex (tensor-core hop)
   uint32_t *Ub16 = nullptr;   // BF16 link bundle of the tile hop, [2 parity][Vh][8 dir][3][3] (re, im) pairs
-  int4 *Ufx = nullptr;        // integer limbs of U64 (fx64.cuh), [V][4][3][3] (re.h, re.l, im.h, im.l)
+  int4 *Ufx = nullptr;        // integer limbs of U64 with the time-boundary sign (layout in fxfield.cuh)
   int4 *Uapefx = nullptr;     // the same of Uape
   double2 *Uape = nullptr;    // APE-smeared copy (spatial links smeared) [V][4][3][3], on first use
   bool have_ape = false;
   std::vector<lqcd::DevBuf> ws;  // named workspaces, grow-only
+  cudaEvent_t fx_ev = nullptr;   // end of the last use of workspace WS_FX, on fx_stream
+  cudaStream_t fx_stream = nullptr;
+  bool fx_used = false;
   lqcd::SloppyState *sloppy = nullptr;
   std::string err;
   int *d_flag = nullptr;      // device error flag scratch
@@ -263,7 +265,7 @@ bool is_device_ptr(const void *p);
 enum WsSlot {
   WS_STAGE_IN = 0, WS_STAGE_OUT, WS_STAGE_AUX,
   WS_F64_VECS, WS_F64_SCAL, WS_F64_PART, WS_F64_FULL,
-  WS_LOOP_PART, WS_GRAD, WS_GRAD2, WS_SMEAR, WS_SMEAR_LINKS,
+  WS_LOOP_PART, WS_GRAD, WS_GRAD2, WS_SMEAR, WS_SMEAR_LINKS, WS_FX,
   WS_COUNT
 };
 
@@ -271,11 +273,6 @@ enum WsSlot {
 int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
                  const double2 *in, size_t in_stride, double2 *out, size_t out_stride, const double2 *A, double cA,
                  const double2 *B, double cB, double cH, const int *active, int nrhs);
-int df_join(lqcd_ctx *ctx, const float4 *in, double2 *out, size_t n, cudaStream_t st);
-// r = b - D x in double-float for the n right-hand sides list[0..n) (host
-// list); rr, bb (host, indexed by right-hand side) receive |r|^2 and |b|^2
-int df_residual(lqcd_ctx *ctx, const float4 *x, const double2 *b, float2 *r, const int *list, int n, double *rr,
-                double *bb, cudaStream_t st);
 int fp64_true_residual(lqcd_ctx *ctx, const double2 *b, const double2 *x, int nrhs, double *rr, double *bb,
                        cudaStream_t st);
 int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, bool dagger,

@@ -9,8 +9,8 @@
 //   * FP32    -- the iterate x and the reliable-update residual
 //               r = b - D_hat x, with FP32 reconstruct-12 links;
 //   * FP64-class -- the outer defect correction: r = b - D x on the full
-//               lattice in double-float arithmetic (a 48-bit significand on the
-//               FP32 units), inner solve D e = r, x += e, until |r| / |b| <= tol.
+//               lattice with 57 bits on the integer units (fxres.cu), inner
+//               solve D e = r, x += e, until |r| / |b| <= tol.
 //
 // Sloppy vectors hold right-hand sides in pairs (RHS 2P and 2P+1): each
 // 16-bit pair is the same real of both members, so after conversion every
@@ -43,10 +43,10 @@
 #include <vector>
 
 #include "internal.cuh"
-#include "df.cuh"
 #include "fpconv.cuh"
 
 #include "sloppy.cuh"
+#include "fxfield.cuh"
 #include "tile_api.cuh"
 
 namespace lqcd {
@@ -1332,25 +1332,22 @@ __device__ __forceinline__ int even_first(const Geom &g, int i) {  // is site 2i
   return ((y + r % g.L[2] + r / g.L[2]) & 1) == 0;
 }
 
-// dst_e / dst_o (FP32 parity fields) = scale[rhs] * src (canonical FP32)
-__global__ void __launch_bounds__(ST) k_cvt32to32_both(Geom g, const float2 *__restrict__ src, F32F de, F32F dodd,
-                                                       const double *scale, const int *list, const int *count,
-                                                       int nbx) {
+// dst = scale[rhs] * src for the FP32 fields of both parities
+__global__ void __launch_bounds__(ST) k_scale32_both(int vh, F32F se, F32F so, F32F de, F32F dodd, const double *scale,
+                                                     const int *list, const int *count, int nbx) {
   const int n_items = *count * nbx;
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     const int rhs = list[w / nbx];
     const int i = (w % nbx) * ST + threadIdx.x;
-    if (i >= g.Vh) continue;
-    const float2 *q = src + ((size_t)rhs * g.V + 2 * (size_t)i) * 12;
+    if (i >= vh) continue;
     const float sc = (float)scale[rhs];
-    const int ef = even_first(g, i);
-    float2 v[12];
+    const size_t o = (size_t)rhs * 6 * vh + i;
+    float4 q[12];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) v[k] = make_float2(q[k].x * sc, q[k].y * sc);
-    (ef ? de : dodd).store(rhs, i, v);
+    for (int k = 0; k < 12; ++k) q[k] = (k < 6 ? se : so).d[o + (size_t)(k % 6) * vh];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) v[k] = make_float2(q[12 + k].x * sc, q[12 + k].y * sc);
-    (ef ? dodd : de).store(rhs, i, v);
+    for (int k = 0; k < 12; ++k)
+      (k < 6 ? de : dodd).d[o + (size_t)(k % 6) * vh] = make_float4(q[k].x * sc, q[k].y * sc, q[k].z * sc, q[k].w * sc);
   }
 }
 
@@ -1389,62 +1386,6 @@ __global__ void __launch_bounds__(ST) k_cvt64to32_both(Geom g, const double2 *__
       }
       ((ef != 0) == (h == 0) ? de : dodd).store(rhs, i, v);
     }
-  }
-}
-
-// x (double-float canonical) += scale[rhs] * (e on even sites, o on odd sites).
-// A block's ST parity-local indices own 2 ST consecutive canonical sites: that
-// contiguous run (ST * 384 B) is staged through shared memory so every global
-// load and store is coalesced.
-constexpr int ACC_SITES = 64;  // parity-local indices per block (48 KiB of shared memory)
-__global__ void __launch_bounds__(ACC_SITES * 2) k_accum_df_both(Geom g, F32F e, F32F o, float4 *x,
-                                                                 const double *scale, const int *list,
-                                                                 const int *count, int nbx) {
-  __shared__ float4 tile[ACC_SITES * 24];
-  const int n_items = *count * nbx;
-  for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
-    const int rhs = list[w / nbx];
-    const int i0 = (w % nbx) * ACC_SITES;
-    const int nloc = min(ACC_SITES, g.Vh - i0);
-    float4 *base = x + ((size_t)rhs * g.V + 2 * (size_t)i0) * 12;
-    constexpr int PER = ACC_SITES * 24 / (ACC_SITES * 2);  // elements per thread of a full tile
-    if (nloc == ACC_SITES) {  // all loads issued before any store: PER requests in flight
-      float4 q[PER];
-#pragma unroll
-      for (int u = 0; u < PER; ++u) q[u] = base[threadIdx.x + u * blockDim.x];
-#pragma unroll
-      for (int u = 0; u < PER; ++u) tile[threadIdx.x + u * blockDim.x] = q[u];
-    } else {
-      for (int k = threadIdx.x; k < nloc * 24; k += blockDim.x) tile[k] = base[k];
-    }
-    __syncthreads();
-    // two threads per parity-local index: one per canonical site of the pair
-    const int li = threadIdx.x >> 1, half = threadIdx.x & 1;
-    if (li < nloc) {
-      const int i = i0 + li;
-      const double scd = scale[rhs];
-      const float sh = (float)scd;
-      const dfl sc{sh, (float)(scd - (double)sh)};
-      const bool even_site = (half == 0) == (even_first(g, i) != 0);
-      float2 v[12];
-      (even_site ? e : o).load(rhs, i, v);
-      float4 *q = tile + (size_t)li * 24 + half * 12;
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        float4 old = q[k];
-        dfl re = df_norm(dfl{old.x, old.z} + sc * dfl{v[k].x, 0.f});
-        dfl im = df_norm(dfl{old.y, old.w} + sc * dfl{v[k].y, 0.f});
-        q[k] = make_float4(re.h, im.h, re.l, im.l);
-      }
-    }
-    __syncthreads();
-    if (nloc == ACC_SITES) {
-#pragma unroll
-      for (int u = 0; u < PER; ++u) base[threadIdx.x + u * blockDim.x] = tile[threadIdx.x + u * blockDim.x];
-    } else {
-      for (int k = threadIdx.x; k < nloc * 24; k += blockDim.x) base[k] = tile[k];
-    }
-    __syncthreads();
   }
 }
 
@@ -1692,8 +1633,8 @@ struct SloppyState {
   uint4 *sd = nullptr;     // 7 sloppy fields (pair or tile layout; same bytes per RHS)
   float2 *sn = nullptr;    // FP16 norms of the pair layout
   float4 *f32 = nullptr;   // 5 FP32 fields
-  float4 *xdf = nullptr;   // the iterate, double-float canonical [cap][V][12]
-  float2 *r32 = nullptr;   // residual b - D x, FP32 canonical (seeds the next inner solve)
+  FxIterate x;             // the iterate, integer limbs
+  float4 *r32 = nullptr;   // residual b - D x, FP32 [2 parity][cap][6][Vh] (seeds the next inner solve)
   char *small = nullptr;
   int *h_counts = nullptr;  // pinned
   // captured graph of four inner iterations, valid while graph_key matches
@@ -1708,7 +1649,8 @@ void sloppy_free(lqcd_ctx *ctx) {
   cudaFree(s->sd);
   cudaFree(s->sn);
   cudaFree(s->f32);
-  cudaFree(s->xdf);
+  cudaFree(s->x.d);
+  cudaFree(s->x.e);
   cudaFree(s->r32);
   cudaFree(s->small);
   if (s->h_counts) cudaFreeHost(s->h_counts);
@@ -1776,10 +1718,11 @@ static int sloppy_alloc(lqcd_ctx *ctx, int nrhs, int gran = 2) {
   cudaFree(s->sd);
   cudaFree(s->sn);
   cudaFree(s->f32);
-  cudaFree(s->xdf);
+  cudaFree(s->x.d);
+  cudaFree(s->x.e);
   cudaFree(s->r32);
   cudaFree(s->small);
-  s->sd = nullptr; s->sn = nullptr; s->f32 = nullptr; s->xdf = nullptr; s->r32 = nullptr;
+  s->sd = nullptr; s->sn = nullptr; s->f32 = nullptr; s->x = FxIterate{}; s->r32 = nullptr;
   s->small = nullptr;
   s->cap = 0;
   const Geom &g = ctx->geom;
@@ -1787,8 +1730,11 @@ static int sloppy_alloc(lqcd_ctx *ctx, int nrhs, int gran = 2) {
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->sd, 7 * pairs * 6 * vh * sizeof(uint4)));
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->sn, 7 * pairs * vh * sizeof(float2)));
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->f32, 5 * (size_t)cap * 6 * vh * sizeof(float4)));
-  LQCD_CUDA_TRY(ctx, cudaMalloc(&s->xdf, (size_t)cap * g.V * 12 * sizeof(float4)));
-  LQCD_CUDA_TRY(ctx, cudaMalloc(&s->r32, (size_t)cap * g.V * 12 * sizeof(float2)));
+  const size_t vpad = 2 * 32 * (size_t)fx_blocks(g.Vh);
+  LQCD_CUDA_TRY(ctx, cudaMalloc(&s->x.d, (size_t)cap * vpad * 12 * sizeof(int4)));
+  LQCD_CUDA_TRY(ctx, cudaMalloc(&s->x.e, (size_t)cap * vpad * sizeof(int)));
+  s->x.cap = cap;
+  LQCD_CUDA_TRY(ctx, cudaMalloc(&s->r32, (size_t)cap * g.V * 6 * sizeof(float4)));
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->small, small_layout(nullptr, cap, part_blocks(g.Vh)).size()));
   // padding right-hand sides of a tile are computed alongside the real ones: start them at zero
   LQCD_CUDA_TRY(ctx, cudaMemset(s->sd, 0, 7 * pairs * 6 * vh * sizeof(uint4)));
@@ -1938,7 +1884,7 @@ struct RunIface {
 //   launch_iters()   a fixed sequence of inner BiCGstab iterations (capturable:
 //                    every kernel reads its work list and counts from device memory)
 //   poll()           after the stream has drained: is the inner solve over?
-//   cycle_end()      odd reconstruction and x += |r| e in FP64
+//   cycle_end()      odd reconstruction and x += |r| e
 template <class Ops>
 struct MixedRun : RunIface {
   using SF = typename Ops::Field;
@@ -1956,9 +1902,9 @@ struct MixedRun : RunIface {
   float kappa = 0.f, k2 = 0.f;
   double delta = 0.05, floor2 = 4e-12;  // (2e-6)^2: inner FP32 target floor, relative to |b_inner|^2
   SF r, rhat, pp, v, s, t, tmp;
-  F32F x32, b32, r32, t32, o32;
+  F32F x32, b32, r32, t32, o32, res[2];  // res: outer residual by parity
   SmallBufs sb;
-  std::vector<double> rr, bb, prev_rel, hscale, hun;
+  std::vector<double> rr, bb, prev_rel, hscale, hun, have;  // have: 1 where the iterate was started
   std::vector<SState> hs;
   std::vector<int> hl, hp, bad, hflags, keep_status;
   int cycle = 0;
@@ -2009,14 +1955,20 @@ struct MixedRun : RunIface {
     hflags.assign(cap, 0);
     keep_status.assign(nrhs, 0);
     for (int k = 0; k < nrhs; ++k) stats[k] = lqcd_solve_stats{0, LQCD_OK, 0.0, 0, 0};
-    const size_t n = (size_t)nrhs * g.V * 12;
-    LQCD_CUDA_TRY(ctx, cudaMemsetAsync(ss->xdf, 0, n * sizeof(float4), st));
+    for (int k = 0; k < 2; ++k) {
+      res[k].d = ss->r32 + (size_t)k * cap * 6 * vh;
+      res[k].vh = vh;
+    }
+    have.assign(cap, 0.0);
     LQCD_CUDA_TRY(ctx, cudaMemsetAsync(sb.counts, 0, 16 * sizeof(int), st));
     return LQCD_OK;
   }
 
-  // the FP64 solution from the double-float iterate
-  int finish() override { return df_join(ctx, ss->xdf, x, (size_t)nrhs * g.V * 12, st); }
+  // the FP64 solution from the iterate's limbs
+  int finish() override {
+    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.scale, have.data(), cap * sizeof(double), cudaMemcpyHostToDevice, st));
+    return fx_join(ctx, ss->x, sb.scale, x, nrhs, st);
+  }
 
   // Autotuning: ms per inner iteration of this layout and launch code, with every
   // right-hand side kept active (zero fields; a target below zero keeps them
@@ -2060,12 +2012,12 @@ struct MixedRun : RunIface {
     return {(double)nrhs, (double)p.precision, (double)p.max_iter, delta, (double)kappa, (double)G, (double)hop_variant,
             (double)Ops::GS, (double)(uintptr_t)ss->sd, (double)(uintptr_t)ss->f32, (double)(uintptr_t)ss->small,
             (double)(uintptr_t)ctx->U16, (double)(uintptr_t)ctx->U32, (double)(uintptr_t)ctx->Ub16,
-            (double)(uintptr_t)ss->xdf, (double)cap};
+            (double)cap};
   }
 
   int cycle_start() override {
-    // at x = 0 the residual is b itself (FP64 norms only); later: double-float
-    // b - D x for the right-hand sides corrected in the previous cycle (the
+    // at x = 0 the residual is b itself (FP64 norms only); later: b - D x on the
+    // integer units for the right-hand sides corrected in the previous cycle (the
     // others' iterates, and so their residuals, have not changed)
     std::vector<int> todo;
     if (cycle == 0) {
@@ -2075,8 +2027,7 @@ struct MixedRun : RunIface {
       todo = hl;
     }
     int rc = cycle == 0 ? fp64_residual_into(ctx, b, nullptr, nullptr, nrhs, rr.data(), bb.data(), st)
-                        : df_residual(ctx, ss->xdf, b, ss->r32, todo.data(), (int)todo.size(), rr.data(),
-                                      bb.data(), st);
+                        : fx_residual(ctx, ss->x, b, res, todo.data(), (int)todo.size(), rr.data(), st);
     if (rc) return rc;
     hl.clear();
     hp.clear();
@@ -2132,7 +2083,7 @@ struct MixedRun : RunIface {
     if (cycle == 0) {
       KL k_cvt64to32_both<<<G, ST, 0, st>>>(g, b, b32, o32, sb.scale, sb.cyc_list, counts + 2, nbx);
     } else {
-      KL k_cvt32to32_both<<<G, ST, 0, st>>>(g, ss->r32, b32, o32, sb.scale, sb.cyc_list, counts + 2, nbx);
+      KL k_scale32_both<<<G, ST, 0, st>>>(vh, res[0], res[1], b32, o32, sb.scale, sb.cyc_list, counts + 2, nbx);
     }
     KL k_hop32x2<EPI_AXPY><<<G, ST, 0, st>>>(g, 0, ctx->U32, o32, b32, b32, b32, 1.f, 0.f, kappa, sb.cyc_list,
                                            counts + 2, nullptr, nbx);
@@ -2235,8 +2186,10 @@ struct MixedRun : RunIface {
     // odd half of the correction: e_o = o32 + kappa H_oe x32; x += |r| e
     KL k_hop32x2<EPI_AXPY><<<G, ST, 0, st>>>(g, 1, ctx->U32, x32, o32, o32, o32, 1.f, 0.f, kappa, sb.cyc_list,
                                            counts + 2, nullptr, nbx);
-    KL k_accum_df_both<<<G, ACC_SITES * 2, 0, st>>>(g, x32, o32, ss->xdf, sb.unscale, sb.cyc_list, counts + 2,
-                                                    (vh + ACC_SITES - 1) / ACC_SITES);
+    int rc = fx_accum(ctx, ss->x, x32, o32, sb.unscale, cycle == 0, sb.cyc_list, counts + 2, G, st);
+    if (rc) return rc;
+    if (cycle == 0)
+      for (int k : hl) have[k] = 1.0;
     LQCD_LAUNCH_CHECK(ctx, "mixed: correction");
     for (int k = 0; k < nrhs; ++k) keep_status[k] = hs[k].status;
     LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(hs.data(), sb.sc, cap * sizeof(SState), cudaMemcpyDeviceToHost, st));

@@ -12,7 +12,7 @@
 #include <cmath>
 
 #include "internal.cuh"
-#include "fx64.cuh"
+#include "fxfield.cuh"
 
 namespace lqcd {
 
@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(128) k_gauss_step(Geom g, const double2 *__res
   const size_t field = (size_t)g.V * 12;
   int c[4];
   coords_full(g, s, c);
+  const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
   long long acc[NR][6];
   int Ea[NR];
   bool bad[NR];
@@ -228,7 +229,8 @@ __global__ void __launch_bounds__(128) k_gauss_step(Geom g, const double2 *__res
     const int sn = fwd ? s + step : s - step;
     const int cj = fwd ? 0 : (int)0x80000000;
     int4 u[9];
-    fx_load_link(Ufx + ((size_t)(fwd ? s : sn) * 4 + mu) * 9, !fwd, u);
+    const int sl = fwd ? s : sn, pl = fwd ? par : 1 - par;  // the link's site
+    fx_load_link(Ufx + fx_link_index(pl, mu, g.Vh, sl >> 1), !fwd, u);
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       const double2 *p = in + (size_t)min(r0 + r, nrhs - 1) * field + (size_t)sn * 12 + spin * 3;
@@ -288,10 +290,19 @@ __global__ void k_gauss_step64(Geom g, const double2 *__restrict__ U, const doub
   for (int k = 0; k < 3; ++k) out[(rhs * g.V + s) * 12 + spin * 3 + k] = cscale(v[k], scale);
 }
 
-// integer limbs of n complex link entries
-__global__ void k_links_fx(const double2 *__restrict__ U, int4 *out, size_t n) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) out[k] = fx_link_entry(U[k].x, U[k].y);
+// integer limbs of the spatial links (layout of fxfield.cuh); thread per (site, mu)
+__global__ void k_links_fx(Geom g, const double2 *__restrict__ U, int4 *out) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = idx >> 2, mu = idx & 3;
+  if (s >= g.V || mu == 3) return;
+  int c[4];
+  coords_full(g, s, c);
+  const int p = (c[0] + c[1] + c[2] + c[3]) & 1;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const double2 u = U[(size_t)idx * 9 + k];
+    out[fx_link_index(p, mu, g.Vh, s >> 1) + 32 * k] = fx_link_entry(u.x, u.y);
+  }
 }
 
 }  // namespace lqcd
@@ -353,9 +364,9 @@ extern "C" int lqcd_smear_gaussian(lqcd_ctx *ctx, const double *in, double *out,
   const double2 *U = ape_links ? ctx->Uape : ctx->U64;
   const int4 *Ufx = ctx->Ufx;
   if (ape_links && ctx->gauge_su3) {  // limbs of the smeared links
-    const size_t nl = (size_t)g.V * 36;
+    const size_t nl = (size_t)fx_blocks(g.Vh) * 8 * 288;
     if (!ctx->Uapefx) LQCD_CUDA_TRY(ctx, cudaMalloc(&ctx->Uapefx, nl * sizeof(int4)));
-    KL k_links_fx<<<(unsigned)((nl + 255) / 256), 256, 0, st>>>(ctx->Uape, ctx->Uapefx, nl);
+    KL k_links_fx<<<(g.V * 4 + 255) / 256, 256, 0, st>>>(g, ctx->Uape, ctx->Uapefx);
     LQCD_LAUNCH_CHECK(ctx, "k_links_fx");
     Ufx = ctx->Uapefx;
   }
