@@ -1637,9 +1637,11 @@ struct SloppyState {
   float4 *r32 = nullptr;   // residual b - D x, FP32 [2 parity][cap][6][Vh] (seeds the next inner solve)
   char *small = nullptr;
   int *h_counts = nullptr;  // pinned
-  // captured graph of four inner iterations, valid while graph_key matches
+  // captured graph of the inner loop, valid while graph_key matches
   cudaGraphExec_t graph = nullptr;
   std::vector<double> graph_key;
+  std::vector<double> direct_key;     // key of the last solve that launched its iterations directly
+  cudaStream_t cap_stream = nullptr;  // the graph is recorded on it, whatever stream it then runs on
   long long graph_kernels = 0;  // kernel launches one replay of the graph makes
 };
 
@@ -1655,6 +1657,7 @@ void sloppy_free(lqcd_ctx *ctx) {
   cudaFree(s->small);
   if (s->h_counts) cudaFreeHost(s->h_counts);
   if (s->graph) cudaGraphExecDestroy(s->graph);
+  if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
   delete s;
   ctx->sloppy = nullptr;
 }
@@ -2312,9 +2315,21 @@ static int mixed_block(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, co
   int rc = run->init();
   if (rc) return rc;
   SloppyState *ss = ctx->sloppy;
-  // the legacy default stream cannot be captured: launch directly there
-  const bool use_graph = !ctx->prof_on && st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread &&
-                         getenv("LQCD_NO_GRAPH") == nullptr;
+  // The graph is recorded on a stream of its own and launched on the caller's, which may
+  // be the default stream.  There the first solve of a configuration launches its
+  // iterations directly: recording a graph takes longer than it saves once, and a
+  // program that solves once on the default stream does not pay for it.
+  bool use_graph = !ctx->prof_on && getenv("LQCD_NO_GRAPH") == nullptr;
+  if (use_graph && (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread)) {
+    const std::vector<double> key = run->graph_key();
+    const bool have = ss->graph && ss->graph_key == key;
+    if (!have && ss->direct_key != key) {
+      ss->direct_key = key;
+      use_graph = false;
+    }
+  }
+  if (use_graph && !ss->cap_stream)
+    LQCD_CUDA_TRY(ctx, cudaStreamCreateWithFlags(&ss->cap_stream, cudaStreamNonBlocking));
   while (!run->done) {
     if (!run->inner) {
       rc = run->cycle_start();
@@ -2328,7 +2343,7 @@ static int mixed_block(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, co
         ss->graph = nullptr;
         cudaGraph_t g = nullptr;
         LQCD_CUDA_TRY(ctx, cudaGraphCreate(&g, 0));
-        cudaError_t e = add_cycle_loop(g, run.get(), st);
+        cudaError_t e = add_cycle_loop(g, run.get(), ss->cap_stream);
         if (e == cudaSuccess) e = cudaGraphInstantiate(&ss->graph, g, 0);
         cudaGraphDestroy(g);
         if (e != cudaSuccess) {
