@@ -1778,7 +1778,11 @@ constexpr int TILE_VARIANT = 5;
 // LQCD_HOP_VARIANT=0..7 in the environment overrides the variant (for tests)
 static int tuned_code(const lqcd_ctx *ctx, int nrhs, int precision) {
   long long key = (long long)nrhs * 8 + precision;
-  int code = 80;
+  // Untuned: the register-capped pair hop on 256 blocks per SM, or as many as there are
+  // items (MixedRun::init).  Against the uncapped one on 8 blocks per SM, 48 right-hand
+  // sides of 24^3 x 48 take 159.6 ms instead of 195.4, an uneven batch of three lattices
+  // 40.6 instead of 45.4; the same results bit for bit.
+  int code = 2561;
   for (auto &kv : ctx->tuned)
     if (kv.first == key) code = kv.second;
   const char *force = getenv("LQCD_HOP_VARIANT");
@@ -1939,6 +1943,7 @@ struct MixedRun : RunIface {
     // tile path: the element-wise kernels use eight 256-thread blocks per SM
     G = num_sms(ctx->device) * (Ops::GS == TR ? 8 : code / 10);
     npairs = (nrhs + 1) / 2;
+    if (Ops::GS == 2) G = (int)std::min<long long>(G, (long long)npairs * nbx);  // no block without an item
     delta = p.delta > 0 ? p.delta : 0.05;
     SF *f[7] = {&r, &rhat, &pp, &v, &s, &t, &tmp};
     for (int k = 0; k < 7; ++k) {
@@ -2318,7 +2323,8 @@ static int mixed_block(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, co
   // The graph is recorded on a stream of its own and launched on the caller's, which may
   // be the default stream.  There the first solve of a configuration launches its
   // iterations directly: recording a graph takes longer than it saves once, and a
-  // program that solves once on the default stream does not pay for it.
+  // program that solves once on the default stream does not pay for it.  12 point
+  // sources of 4^4: 1.70 -> 1.20 ms, 17 sources of 8^3 x 16 (FP16): 2.94 -> 2.00 ms.
   bool use_graph = !ctx->prof_on && getenv("LQCD_NO_GRAPH") == nullptr;
   if (use_graph && (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread)) {
     const std::vector<double> key = run->graph_key();
