@@ -166,7 +166,7 @@ __global__ void k_plaquette(const double2 *__restrict__ U, Geom g, double *parti
         for (int i = 0; i < 3; ++i)
           for (int j = 0; j < 3; ++j) {
             double2 t = make_double2(0, 0);
-            for (int k = 0; k < 3; ++k) t = cadd(t, dmul(a[i * 3 + k], b[k * 3 + j]));
+            for (int k = 0; k < 3; ++k) t = cmac(t, a[i * 3 + k], b[k * 3 + j]);
             ab[i][j] = t;
           }
         for (int i = 0; i < 3; ++i)
@@ -175,7 +175,7 @@ __global__ void k_plaquette(const double2 *__restrict__ U, Geom g, double *parti
             for (int k = 0; k < 3; ++k) {
               double2 cj = cc[j * 3 + k];
               cj.y = -cj.y;
-              t = cadd(t, dmul(ab[i][k], cj));
+              t = cmac(t, ab[i][k], cj);
             }
             abc[i][j] = t;
           }
@@ -183,7 +183,7 @@ __global__ void k_plaquette(const double2 *__restrict__ U, Geom g, double *parti
           for (int k = 0; k < 3; ++k) {
             double2 dk = d[i * 3 + k];
             dk.y = -dk.y;
-            acc += dmul(abc[i][k], dk).x;
+            acc = fma(-abc[i][k].y, dk.y, fma(abc[i][k].x, dk.x, acc));
           }
       }
   }
