@@ -250,7 +250,6 @@ int lqcd_destroy(lqcd_ctx *ctx) {
   cudaFree(ctx->Ub16);
   cudaFree(ctx->Uape);
   cudaFree(ctx->Ufx);
-  cudaFree(ctx->Uapefx);
   if (ctx->fx_ev) cudaEventDestroy(ctx->fx_ev);
   cudaFree(ctx->d_flag);
   cudaFree(ctx->d_prof);

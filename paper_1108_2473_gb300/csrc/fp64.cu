@@ -222,39 +222,48 @@ __global__ void __launch_bounds__(128, 4) k_hop64_fxf(Geom g, int p_out, const d
   hop64_store(v, (size_t)rhs * out_stride + s * 12 + hs * 3, out, A, cA, B, cB, cH);
 }
 
-// Workspace of integer limbs for n_par parities of up to *chunk right-hand sides, or
-// null (then the caller takes FP64 arithmetic, as for links that are not SU(3), which
-// may be of any size): as many as keep it in L2 (FX_WS_BYTES), at least one.  Not while the stream is being captured, when nothing
-// may be allocated.  The workspace is shared by the context's streams: a call waits
-// for the last one's event, and fx_workspace_done records its own.
-constexpr size_t FX_WS_BYTES = 96u << 20;
-static char *fx_workspace(lqcd_ctx *ctx, int nrhs, int n_par, int *chunk, cudaStream_t st) {
+static bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  const size_t per = (size_t)n_par * fx_blocks(ctx->geom.Vh) * 32 * (12 * sizeof(int4) + sizeof(int));
-  *chunk = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FX_WS_BYTES / per));
-  int rc = LQCD_OK;
-  void *w = workspace(ctx, WS_FX, per * *chunk, &rc);
-  if (!w) return nullptr;
+  const bool err = cudaStreamIsCapturing(st, &cap) != cudaSuccess;
+  if (err) cudaGetLastError();
+  return err || cap != cudaStreamCaptureStatusNone;
+}
+// The workspaces of integer limbs are shared by the context's streams: a call that uses
+// one waits for the event of the last (fx_enter) and records its own (fx_leave).  Under
+// capture neither does anything: the graph's order is its program's.
+bool fx_enter(lqcd_ctx *ctx, cudaStream_t st) {
+  if (capturing(st)) return true;
   if (!ctx->fx_ev && cudaEventCreateWithFlags(&ctx->fx_ev, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     ctx->fx_ev = nullptr;
-    return nullptr;
+    return false;
   }
   if (ctx->fx_used && ctx->fx_stream != st && cudaStreamWaitEvent(st, ctx->fx_ev, 0) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    return false;
   }
-  return (char *)w;
+  return true;
 }
-static int fx_workspace_done(lqcd_ctx *ctx, cudaStream_t st) {
+int fx_leave(lqcd_ctx *ctx, cudaStream_t st) {
+  if (capturing(st)) return LQCD_OK;
   LQCD_CUDA_TRY(ctx, cudaEventRecord(ctx->fx_ev, st));
   ctx->fx_used = true;
   ctx->fx_stream = st;
   return LQCD_OK;
+}
+
+// Workspace of integer limbs for n_par parities of up to *chunk right-hand sides, or
+// null (then the caller takes FP64 arithmetic, as for links that are not SU(3), which
+// may be of any size): as many as keep it in L2 (FX_WS_BYTES), at least one.  Not while
+// the stream is being captured, when nothing may be allocated.
+constexpr size_t FX_WS_BYTES = 96u << 20;
+static char *fx_workspace(lqcd_ctx *ctx, int nrhs, int n_par, int *chunk, cudaStream_t st) {
+  if (capturing(st)) return nullptr;
+  const size_t per = (size_t)n_par * fx_blocks(ctx->geom.Vh) * 32 * (12 * sizeof(int4) + sizeof(int));
+  *chunk = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FX_WS_BYTES / per));
+  int rc = LQCD_OK;
+  void *w = workspace(ctx, WS_FX, per * *chunk, &rc);
+  return w && fx_enter(ctx, st) ? (char *)w : nullptr;
 }
 // one launch; fx: the input as integer limbs, or null
 static int launch_hop64_one(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
@@ -315,7 +324,7 @@ int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool o
                               A ? A + o : nullptr, cA, B ? B + o : nullptr, cB, cH, act, n, &f);
     if (rc) return rc;
   }
-  return fx_workspace_done(ctx, st);
+  return fx_leave(ctx, st);
 }
 
 int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, bool dagger, cudaStream_t st) {
@@ -342,7 +351,7 @@ int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, b
       if (rc) return rc;
     }
   }
-  return w ? fx_workspace_done(ctx, st) : LQCD_OK;
+  return w ? fx_leave(ctx, st) : LQCD_OK;
 }
 
 // --------------------------------------------------------- layout changes

@@ -61,62 +61,43 @@ template <int SH> __device__ __forceinline__ long long fx_int(double v, int E, i
 }
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return c + (long long)a * b; }
 
-// X = U h for a colour vector h (re, im of three colours).  U^+ h is
-// conj(U^T conj(h)): the callers load the transpose and conjugate on both sides.
-__device__ __forceinline__ void fx_su3(const int4 u[9], const long long h[6], long long X[6]) {
-  int xh[6], xl[6], nh[3], nl[3];
+// X = U h (FWD) or U^+ h for a colour vector h in limbs (rh, rl the real, ih, il the
+// imaginary parts): 108 integer multiply-adds
+template <bool FWD>
+__device__ __forceinline__ void fx_su3(const int4 u[9], const int rh[3], const int rl[3], const int ih[3],
+                                       const int il[3], long long X[6]) {
+  int nh[3], nl[3];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) fx_split(h[k], xh[k], xl[k]);
-#pragma unroll
-  for (int b = 0; b < 3; ++b) {
-    nh[b] = -xh[2 * b + 1];
-    nl[b] = -xl[2 * b + 1];
+  for (int k = 0; k < 3; ++k) {
+    nh[k] = FWD ? -ih[k] : -rh[k];  // the part that enters with a minus sign
+    nl[k] = FWD ? -il[k] : -rl[k];
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    long long ar = 0, br = 0, ai = 0, bi = 0;
+    long long ar = 0, br = 1ll << 28, ai = 0, bi = 1ll << 28;  // b: rounded when shifted
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const int4 w = u[a * 3 + b];
-      const int rh = xh[2 * b], rl = xl[2 * b], ih = xh[2 * b + 1], il = xl[2 * b + 1];
-      ar = fx_mad(w.x, rh, ar);
-      br = fx_mad(w.x, rl, br);
-      br = fx_mad(w.y, rh, br);
-      ar = fx_mad(w.z, nh[b], ar);
-      br = fx_mad(w.z, nl[b], br);
-      br = fx_mad(w.w, nh[b], br);
-      ai = fx_mad(w.x, ih, ai);
-      bi = fx_mad(w.x, il, bi);
-      bi = fx_mad(w.y, ih, bi);
-      ai = fx_mad(w.z, rh, ai);
-      bi = fx_mad(w.z, rl, bi);
-      bi = fx_mad(w.w, rh, bi);
+      const int4 m = FWD ? u[a * 3 + b] : u[b * 3 + a];  // U, or U^+ = conj of the transpose
+      const int ph = FWD ? nh[b] : ih[b], pl = FWD ? nl[b] : il[b];
+      const int qh = FWD ? rh[b] : nh[b], ql = FWD ? rl[b] : nl[b];
+      ar = fx_mad(m.x, rh[b], ar);
+      br = fx_mad(m.x, rl[b], br);
+      br = fx_mad(m.y, rh[b], br);
+      ar = fx_mad(m.z, ph, ar);
+      br = fx_mad(m.z, pl, br);
+      br = fx_mad(m.w, ph, br);
+      ai = fx_mad(m.x, ih[b], ai);
+      bi = fx_mad(m.x, il[b], bi);
+      bi = fx_mad(m.y, ih[b], bi);
+      ai = fx_mad(m.z, qh, ai);
+      bi = fx_mad(m.z, ql, bi);
+      bi = fx_mad(m.w, qh, bi);
     }
-    X[2 * a] = ar + ((br + (1ll << 28)) >> 29);
-    X[2 * a + 1] = ai + ((bi + (1ll << 28)) >> 29);
+    X[2 * a] = ar + (br >> 29);
+    X[2 * a + 1] = ai + (bi >> 29);
   }
-}
-// the link at w (entries 32 apart), or its transpose
-__device__ __forceinline__ void fx_load_link(const int4 *__restrict__ w, bool transpose, int4 u[9]) {
-  const int sa = transpose ? 32 : 96, sb = transpose ? 96 : 32;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) u[a * 3 + b] = w[a * sa + b * sb];
 }
 __device__ __forceinline__ long long fx_negif(long long v, long long mask) { return (v ^ mask) - mask; }
-
-// acc (N sums at exponent Ea) brought to an exponent of at least E; returns the
-// shift that aligns a contribution at exponent E with it
-template <int N> __device__ __forceinline__ int fx_align(long long acc[N], int &Ea, int E) {
-  if (E > Ea) {
-    const int d = min(E - Ea, 63);
-#pragma unroll
-    for (int k = 0; k < N; ++k) acc[k] >>= d;
-    Ea = E;
-  }
-  return min(Ea - E, 63);
-}
 
 // acc 2^(Ea - 1075 - SH) as FP64
 template <int SH> __device__ __forceinline__ double fx_double(long long acc, int Ea) {

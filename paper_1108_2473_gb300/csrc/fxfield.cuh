@@ -72,7 +72,7 @@ __device__ __forceinline__ void fxf_dir(int j, int n, const int4 *__restrict__ w
   int4 u[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) u[k] = w[32 * k];
-  int rh[3], rl[3], ih[3], il[3], nh[3], nl[3];
+  int rh[3], rl[3], ih[3], il[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const int4 a = q[32 * (3 * HS + k)];
@@ -89,32 +89,13 @@ __device__ __forceinline__ void fxf_dir(int j, int n, const int4 *__restrict__ w
       ih[k] = SG > 0 ? a.z + b.z : a.z - b.z;
       il[k] = SG > 0 ? a.w + b.w : a.w - b.w;
     }
-    nh[k] = FWD ? -ih[k] : -rh[k];  // the part that enters with a minus sign
-    nl[k] = FWD ? -il[k] : -rl[k];
   }
   const int d = min(Em - En, 63);
+  long long X[6];
+  fx_su3<FWD>(u, rh, rl, ih, il, X);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    long long ar = 0, br = 1ll << 28, ai = 0, bi = 1ll << 28;  // b: rounded when shifted
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int4 m = FWD ? u[a * 3 + b] : u[b * 3 + a];  // U, or U^+ = conj of the transpose
-      const int ph = FWD ? nh[b] : ih[b], pl = FWD ? nl[b] : il[b];
-      const int qh = FWD ? rh[b] : nh[b], ql = FWD ? rl[b] : nl[b];
-      ar = fx_mad(m.x, rh[b], ar);
-      br = fx_mad(m.x, rl[b], br);
-      br = fx_mad(m.y, rh[b], br);
-      ar = fx_mad(m.z, ph, ar);
-      br = fx_mad(m.z, pl, br);
-      br = fx_mad(m.w, ph, br);
-      ai = fx_mad(m.x, ih[b], ai);
-      bi = fx_mad(m.x, il[b], bi);
-      bi = fx_mad(m.y, ih[b], bi);
-      ai = fx_mad(m.z, qh, ai);
-      bi = fx_mad(m.z, ql, bi);
-      bi = fx_mad(m.w, qh, bi);
-    }
-    const long long xr = (ar + (br >> 29)) >> d, xi = (ai + (bi >> 29)) >> d;
+    const long long xr = X[2 * a] >> d, xi = X[2 * a + 1] >> d;
     up[2 * a] += xr;
     up[2 * a + 1] += xi;
     const long long yr = VAR ? fx_negif(xr, neg) : xr, yi = VAR ? fx_negif(xi, neg) : xi;

@@ -191,11 +191,10 @@ struct lqcd_ctx {
   float2 *Utf = nullptr;      // tf32-rounded FP32, [2 parity][4 mu][Vh][3][3] complex (tensor-core hop)
   uint32_t *Ub16 = nullptr;   // BF16 link bundle of the tile hop, [2 parity][Vh][8 dir][3][3] (re, im) pairs
   int4 *Ufx = nullptr;        // integer limbs of U64 with the time-boundary sign (layout in fxfield.cuh)
-  int4 *Uapefx = nullptr;     // the same of Uape
   double2 *Uape = nullptr;    // APE-smeared copy (spatial links smeared) [V][4][3][3], on first use
   bool have_ape = false;
   std::vector<lqcd::DevBuf> ws;  // named workspaces, grow-only
-  cudaEvent_t fx_ev = nullptr;   // end of the last use of workspace WS_FX, on fx_stream
+  cudaEvent_t fx_ev = nullptr;   // end of the last use of a workspace of limbs, on fx_stream
   cudaStream_t fx_stream = nullptr;
   bool fx_used = false;
   lqcd::SloppyState *sloppy = nullptr;
@@ -247,6 +246,8 @@ extern std::atomic<long long> g_launches;
 int set_error(lqcd_ctx *ctx, int code, const char *fmt, ...);
 int cuda_error(lqcd_ctx *ctx, cudaError_t e, const char *where);
 void *workspace(lqcd_ctx *ctx, int slot, size_t bytes, int *status);
+bool fx_enter(lqcd_ctx *ctx, cudaStream_t st);  // around the use of a workspace of limbs
+int fx_leave(lqcd_ctx *ctx, cudaStream_t st);
 bool is_device_ptr(const void *p);
 
 #define LQCD_CUDA_TRY(ctx, call)                         \
@@ -265,7 +266,7 @@ bool is_device_ptr(const void *p);
 enum WsSlot {
   WS_STAGE_IN = 0, WS_STAGE_OUT, WS_STAGE_AUX,
   WS_F64_VECS, WS_F64_SCAL, WS_F64_PART, WS_F64_FULL,
-  WS_LOOP_PART, WS_GRAD, WS_GRAD2, WS_SMEAR, WS_SMEAR_LINKS, WS_FX,
+  WS_LOOP_PART, WS_GRAD, WS_GRAD2, WS_SMEAR, WS_SMEAR_LINKS, WS_SMEAR_FX, WS_FX,
   WS_COUNT
 };
 

@@ -88,3 +88,51 @@ def test_gaussian_step_over_magnitudes(dims, n, spread, scale):
         L.lqcd_smear_gaussian(h, x, out, alpha=0.7, n_iter=1)
         ref = gaussian_smear(U, q, 0.7, 1)
         assert np.all(np.abs(to_np(out, dims) - ref) <= TOL * _local_max(q) + 1e-320)
+
+
+@pytest.mark.parametrize("dims", DIMS)
+@pytest.mark.parametrize("alpha", [4.0, -0.3, 0.0, 1e-310])
+def test_gaussian_steps_over_coefficients(dims, alpha):
+    """Five normalised steps: zero and negative alpha, and a subnormal one, which has no
+    integer form and takes FP64 arithmetic."""
+    U = haar_su3_field(dims, 8)
+    q = _field(dims, 2, 19, 0, 1.0)
+    q[1] = 0.0
+    q[1, 1, 1, 1, 1, 2, 0] = 1.0  # a point source: most neighbours are zero
+    scale = 1.0 / (1.0 + 6.0 * alpha)
+    with lattice(dims, U, 0.13) as (L, h):
+        x = to_dev(q.reshape(2, -1, 4, 3))
+        out = torch.empty_like(x)
+        L.lqcd_smear_gaussian(h, x, out, alpha=alpha, n_iter=5, normalise=True)
+        got = to_np(out, dims)
+    ref = gaussian_smear(U, q, alpha, 5) * scale**5
+    # a few FP64 roundings of the largest intermediate value per step, in the oracle and here
+    assert np.all(np.abs(got - ref) <= 5 * TOL * max(1.0, (1.0 + 6.0 * abs(alpha)) * abs(scale)) ** 5 * np.abs(q).max())
+
+
+@pytest.mark.parametrize("alpha", [4.0, 0.6])
+def test_gaussian_steps_keep_more_than_fp64(alpha):
+    """25 normalised steps against extended precision.  A step rounds by at most 2^-55 of
+    the vector (58-bit limbs, sums of six products) and the result by 2^-53 once: 8.1e-16
+    in the 2-norm even if all errors line up.  The rounding of 1 / (1 + 6 alpha) to FP64
+    alone would give up to 25 * 2^-53 = 2.8e-15."""
+    dims = (4, 4, 4, 4)
+    U = haar_su3_field(dims, 9)
+    q = gaussian_spinors(dims, 1, 23)
+    with lattice(dims, U, 0.13) as (L, h):
+        x = to_dev(q.reshape(1, -1, 4, 3))
+        out = torch.empty_like(x)
+        L.lqcd_smear_gaussian(h, x, out, alpha=alpha, n_iter=25, normalise=True)
+        got = to_np(out, dims)
+    Q = np.clongdouble
+    u, ref, a = U.astype(Q), q[0].astype(Q), np.longdouble(alpha)
+    for _ in range(25):
+        hq = 0
+        for mu in range(3):
+            um = u[..., mu, :, :]
+            fwd = (um[..., None, :, :] * np.roll(ref, -1, 3 - mu)[..., None, :]).sum(-1)
+            bwd = (np.conj(np.swapaxes(um, -1, -2))[..., None, :, :] * ref[..., None, :]).sum(-1)
+            hq = hq + fwd + np.roll(bwd, 1, 3 - mu)
+        ref = (ref + a * hq) / (1 + 6 * a)
+    d = got[0].astype(Q) - ref
+    assert float(np.sqrt((np.abs(d) ** 2).sum() / (np.abs(ref) ** 2).sum())) < 8.1e-16
