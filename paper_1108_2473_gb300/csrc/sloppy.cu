@@ -332,12 +332,46 @@ __device__ __forceinline__ void pair_reduce_store(float2 re, float2 im, float2 n
   __syncthreads();
 }
 
-// FP32 hopping term: out = cA A + cB B + cH (H in) at the sites of parity p_out.
-// EPI_PLAIN: A, B unused.  EPI_AXPY: B unused.  EPI_RES: partial |out|^2.
+// One site of the FP32 hopping term for right-hand sides rhs[0], rhs[1]: out = cA A +
+// cB B + cH acc, acc = H in.  EPI_PLAIN: A, B unused.  EPI_AXPY: B unused.  EPI_RES: returns
+// |out|^2 of each.  two: false if rhs[1] only repeats rhs[0], and is not stored.
+template <int EPI>
+__device__ __forceinline__ float2 hop32x2_store(const float2 acc[2][4][3], int i, const F32F &out, const F32F &A,
+                                                const F32F &B, float cA, float cB, float cH, const int rhs[2],
+                                                bool two) {
+  float2 red = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    float2 o[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[k] = make_float2(cH * acc[r][k / 3][k % 3].x, cH * acc[r][k / 3][k % 3].y);
+    if (EPI != EPI_PLAIN) {
+      float2 a[12];
+      A.load(rhs[r], i, a);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) o[k] = make_float2(fmaf(cA, a[k].x, o[k].x), fmaf(cA, a[k].y, o[k].y));
+    }
+    if (EPI == EPI_RES) {
+      float2 b[12];
+      B.load(rhs[r], i, b);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) o[k] = make_float2(fmaf(cB, b[k].x, o[k].x), fmaf(cB, b[k].y, o[k].y));
+    }
+    if (r == 0 || two) out.store(rhs[r], i, o);
+    if (EPI == EPI_RES) {
+      float nn = 0.f;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) nn += o[k].x * o[k].x + o[k].y * o[k].y;
+      (r == 0 ? red.x : red.y) = nn;
+    }
+  }
+  return red;
+}
+
 // The FP32 hopping term on two right-hand sides per thread (list entries 2j and
 // 2j + 1; with an odd count the last thread recomputes entry 2j for its second
 // slot and stores nothing for it), which halves the link loads and the
-// reconstruction of the third link row per right-hand side.
+// reconstruction of the third link row per right-hand side.  EPI_RES: partial |out|^2.
 template <int EPI>
 __global__ void __launch_bounds__(ST, 4) k_hop32x2(Geom g, int p_out, const float4 *links, F32F in, F32F out, F32F A,
                                                 F32F B, float cA, float cB, float cH, const int *list,
@@ -355,40 +389,12 @@ __global__ void __launch_bounds__(ST, 4) k_hop32x2(Geom g, int p_out, const floa
       coords_of(g, p_out, i, c);
       float2 acc[2][4][3];
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 3; ++b) acc[r][a][b] = make_float2(0.f, 0.f);
+      for (int k = 0; k < 24; ++k) acc[k / 12][k / 3 % 4][k % 3] = make_float2(0.f, 0.f);
       hop_dir32n<0, 2>(g, p_out, c, i, in, rhs, links, acc);
       hop_dir32n<1, 2>(g, p_out, c, i, in, rhs, links, acc);
       hop_dir32n<2, 2>(g, p_out, c, i, in, rhs, links, acc);
       hop_dir32n<3, 2>(g, p_out, c, i, in, rhs, links, acc);
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        float2 o[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) o[k] = make_float2(cH * acc[r][k / 3][k % 3].x, cH * acc[r][k / 3][k % 3].y);
-        if (EPI != EPI_PLAIN) {
-          float2 a[12];
-          A.load(rhs[r], i, a);
-#pragma unroll
-          for (int k = 0; k < 12; ++k) o[k] = make_float2(fmaf(cA, a[k].x, o[k].x), fmaf(cA, a[k].y, o[k].y));
-        }
-        if (EPI == EPI_RES) {
-          float2 b[12];
-          B.load(rhs[r], i, b);
-#pragma unroll
-          for (int k = 0; k < 12; ++k) o[k] = make_float2(fmaf(cB, b[k].x, o[k].x), fmaf(cB, b[k].y, o[k].y));
-        }
-        if (r == 0 || two) out.store(rhs[r], i, o);
-        if (EPI == EPI_RES) {
-          float nn = 0.f;
-#pragma unroll
-          for (int k = 0; k < 12; ++k) nn += o[k].x * o[k].x + o[k].y * o[k].y;
-          (r == 0 ? red.x : red.y) = nn;
-        }
-      }
+      red = hop32x2_store<EPI>(acc, i, out, A, B, cA, cB, cH, rhs, two);
     }
     if (EPI == EPI_RES)  // an odd last entry has only one right-hand side (its second sum is not stored)
       pair_reduce_store<1, SUM_NORM>(red, red, red, part + (size_t)rhs[0] * nbx + sb,
@@ -1157,7 +1163,138 @@ __device__ __forceinline__ CP cp_fms(const CP &s, const CP &z, const CP &a) {  /
   return CP{F2(s.im, z.im, S2(a.re, M2(s.re, z.re))), S2(a.im, F2(s.re, z.im, M2(s.im, z.re)))};
 }
 
+// One site of the solver's vector updates for pair P, whose members' scalars are s0, s1
+// and flags f0, f1.
 // p = r + beta (p - omega v); members flagged for restart take rhat = r, p = r.
+template <class SP>
+__device__ __forceinline__ void pair_p_site(const SState &s0, const SState &s1, const SP &r, const SP &rhat,
+                                            const SP &p, const SP &v, int P, int i) {
+  const bool re0 = s0.restart, re1 = s1.restart;
+  float2 rv[24], pv[24];
+  load_scaled(r, P, i, rv);
+  if (!(re0 && re1)) {
+    float2 vv[24];
+    load_scaled(p, P, i, pv);
+    load_scaled(v, P, i, vv);
+    const CP be = scal_pair(s0.beta, s1.beta);
+    const CP om = scal_pair(s0.omega, s1.omega);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      CP t = cp_fms(om, CP{vv[2 * k], vv[2 * k + 1]}, CP{pv[2 * k], pv[2 * k + 1]});
+      CP n = cp_fma(be, t, CP{rv[2 * k], rv[2 * k + 1]});
+      pv[2 * k] = n.re;
+      pv[2 * k + 1] = n.im;
+    }
+  }
+  if (re0 || re1) {
+#pragma unroll
+    for (int k = 0; k < 24; ++k) pv[k] = sel2(re0, re1, rv[k], pv[k]);
+    store_members(rhat, P, i, rv, re0, re1);
+  }
+  store_pair(p, P, i, pv);
+}
+// s = r - alpha v
+template <class SP>
+__device__ __forceinline__ void pair_s_site(const SState &s0, const SState &s1, const SP &r, const SP &v, const SP &s,
+                                            int P, int i) {
+  const CP al = scal_pair(s0.alpha, s1.alpha);
+  float2 rv[24], vv[24];
+  load_scaled(r, P, i, rv);
+  load_scaled(v, P, i, vv);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    CP n = cp_fms(al, CP{vv[2 * k], vv[2 * k + 1]}, CP{rv[2 * k], rv[2 * k + 1]});
+    rv[2 * k] = n.re;
+    rv[2 * k + 1] = n.im;
+  }
+  store_pair(s, P, i, rv);
+}
+// x += alpha p + omega s (FP32 x, active members only); r = s - omega t; the site's
+// terms of <rhat, r> and |r|^2 per member
+template <class SP>
+__device__ __forceinline__ void pair_xr_site(const SState &s0, const SState &s1, int f0, int f1, const F32F &x,
+                                             const SP &p, const SP &s, const SP &t, const SP &r, const SP &rhat, int P,
+                                             int i, float2 &sre, float2 &sim, float2 &snn) {
+  const bool a0 = f0 & FLAG_ACTIVE, a1 = f1 & FLAG_ACTIVE;
+  const CP al = scal_pair(s0.alpha, s1.alpha);
+  const CP om = scal_pair(s0.omega, s1.omega);
+  float2 pv[24], sv[24], tv[24];
+  load_scaled(p, P, i, pv);
+  load_scaled(s, P, i, sv);
+  load_scaled(t, P, i, tv);
+  float2 x0[12], x1[12];
+  if (a0) x.load(2 * P, i, x0);
+  if (a1) x.load(2 * P + 1, i, x1);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    CP xk{make_float2(a0 ? x0[k].x : 0.f, a1 ? x1[k].x : 0.f), make_float2(a0 ? x0[k].y : 0.f, a1 ? x1[k].y : 0.f)};
+    xk = cp_fma(al, CP{pv[2 * k], pv[2 * k + 1]}, xk);
+    xk = cp_fma(om, CP{sv[2 * k], sv[2 * k + 1]}, xk);
+    x0[k] = make_float2(xk.re.x, xk.im.x);
+    x1[k] = make_float2(xk.re.y, xk.im.y);
+    CP rn = cp_fms(om, CP{tv[2 * k], tv[2 * k + 1]}, CP{sv[2 * k], sv[2 * k + 1]});
+    sv[2 * k] = rn.re;
+    sv[2 * k + 1] = rn.im;
+  }
+  if (a0) x.store(2 * P, i, x0);
+  if (a1) x.store(2 * P + 1, i, x1);
+  store_pair(r, P, i, sv);
+  load_scaled(rhat, P, i, pv);
+  float2 re = make_float2(0.f, 0.f), ip = re, im = re, nn = re;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    re = F2(pv[2 * k], sv[2 * k], re);
+    re = F2(pv[2 * k + 1], sv[2 * k + 1], re);
+    ip = F2(pv[2 * k], sv[2 * k + 1], ip);
+    im = F2(pv[2 * k + 1], sv[2 * k], im);
+    nn = F2(sv[2 * k], sv[2 * k], nn);
+    nn = F2(sv[2 * k + 1], sv[2 * k + 1], nn);
+  }
+  sre = re;
+  sim = S2(ip, im);
+  snn = nn;
+}
+// members flagged FLAG_RU: r = src (FP32), optionally x = 0; the site's terms of
+// <rhat, r> (or <r, r>) and |r|^2 per member
+template <class SP>
+__device__ __forceinline__ void pair_copy_site(int f0, int f1, const F32F &src, const SP &r, const SP &rhat,
+                                               bool use_rhat, const F32F &x, bool zero_x, int P, int i, float2 &sre,
+                                               float2 &sim, float2 &snn) {
+  const bool w0 = f0 & FLAG_RU, w1 = f1 & FLAG_RU;
+  float2 e0[12], e1[12], v[24];
+  if (w0) src.load(2 * P, i, e0);
+  if (w1) src.load(2 * P + 1, i, e1);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    v[2 * k] = make_float2(w0 ? e0[k].x : 0.f, w1 ? e1[k].x : 0.f);
+    v[2 * k + 1] = make_float2(w0 ? e0[k].y : 0.f, w1 ? e1[k].y : 0.f);
+  }
+  store_members(r, P, i, v, w0, w1);
+  if (zero_x) {
+    float2 z[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) z[k] = make_float2(0.f, 0.f);
+    if (w0) x.store(2 * P, i, z);
+    if (w1) x.store(2 * P + 1, i, z);
+  }
+  float2 q[24];
+  if (use_rhat) load_scaled(rhat, P, i, q);
+  float2 re = make_float2(0.f, 0.f), ip = re, im = re, nn = re;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const float2 qr = use_rhat ? q[2 * k] : v[2 * k], qi = use_rhat ? q[2 * k + 1] : v[2 * k + 1];
+    re = F2(qr, v[2 * k], re);
+    re = F2(qi, v[2 * k + 1], re);
+    ip = F2(qr, v[2 * k + 1], ip);
+    im = F2(qi, v[2 * k], im);
+    nn = F2(v[2 * k], v[2 * k], nn);
+    nn = F2(v[2 * k + 1], v[2 * k + 1], nn);
+  }
+  sre = re;
+  sim = S2(ip, im);
+  snn = nn;
+}
+
 template <class SP>
 __global__ void __launch_bounds__(ST) k_pair_p(int vh, const SState *sc, SP r, SP rhat, SP p, SP v,
                                                const int *plist, const int *pcount, int nbx) {
@@ -1165,34 +1302,10 @@ __global__ void __launch_bounds__(ST) k_pair_p(int vh, const SState *sc, SP r, S
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     const int P = plist[w / nbx];
     const int i = (w % nbx) * ST + threadIdx.x;
-    if (i >= vh) continue;
-    const bool re0 = sc[2 * P].restart, re1 = sc[2 * P + 1].restart;
-    float2 rv[24], pv[24];
-    load_scaled(r, P, i, rv);
-    if (!(re0 && re1)) {
-      float2 vv[24];
-      load_scaled(p, P, i, pv);
-      load_scaled(v, P, i, vv);
-      const CP be = scal_pair(sc[2 * P].beta, sc[2 * P + 1].beta);
-      const CP om = scal_pair(sc[2 * P].omega, sc[2 * P + 1].omega);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        CP t = cp_fms(om, CP{vv[2 * k], vv[2 * k + 1]}, CP{pv[2 * k], pv[2 * k + 1]});
-        CP n = cp_fma(be, t, CP{rv[2 * k], rv[2 * k + 1]});
-        pv[2 * k] = n.re;
-        pv[2 * k + 1] = n.im;
-      }
-    }
-    if (re0 || re1) {
-#pragma unroll
-      for (int k = 0; k < 24; ++k) pv[k] = sel2(re0, re1, rv[k], pv[k]);
-      store_members(rhat, P, i, rv, re0, re1);
-    }
-    store_pair(p, P, i, pv);
+    if (i < vh) pair_p_site(sc[2 * P], sc[2 * P + 1], r, rhat, p, v, P, i);
   }
 }
 
-// s = r - alpha v
 template <class SP>
 __global__ void __launch_bounds__(ST) k_pair_s(int vh, const SState *sc, SP r, SP v, SP s, const int *plist,
                                                const int *pcount, int nbx) {
@@ -1200,23 +1313,10 @@ __global__ void __launch_bounds__(ST) k_pair_s(int vh, const SState *sc, SP r, S
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     const int P = plist[w / nbx];
     const int i = (w % nbx) * ST + threadIdx.x;
-    if (i >= vh) continue;
-    const CP al = scal_pair(sc[2 * P].alpha, sc[2 * P + 1].alpha);
-    float2 rv[24], vv[24];
-    load_scaled(r, P, i, rv);
-    load_scaled(v, P, i, vv);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      CP n = cp_fms(al, CP{vv[2 * k], vv[2 * k + 1]}, CP{rv[2 * k], rv[2 * k + 1]});
-      rv[2 * k] = n.re;
-      rv[2 * k + 1] = n.im;
-    }
-    store_pair(s, P, i, rv);
+    if (i < vh) pair_s_site(sc[2 * P], sc[2 * P + 1], r, v, s, P, i);
   }
 }
 
-// x += alpha p + omega s (FP32 x, active members only); r = s - omega t;
-// partials <rhat, r> and |r|^2 per member
 template <class SP>
 __global__ void __launch_bounds__(ST) k_pair_xr(int vh, const SState *sc, const int *flags, F32F x, SP p, SP s, SP t,
                                                 SP r, SP rhat, const int *plist, const int *pcount, D4S *part,
@@ -1226,53 +1326,13 @@ __global__ void __launch_bounds__(ST) k_pair_xr(int vh, const SState *sc, const 
     const int P = plist[w / nbx], sb = w % nbx;
     const int i = sb * ST + threadIdx.x;
     float2 sre = make_float2(0.f, 0.f), sim = sre, snn = sre;
-    if (i < vh) {
-      const bool a0 = flags[2 * P] & FLAG_ACTIVE, a1 = flags[2 * P + 1] & FLAG_ACTIVE;
-      const CP al = scal_pair(sc[2 * P].alpha, sc[2 * P + 1].alpha);
-      const CP om = scal_pair(sc[2 * P].omega, sc[2 * P + 1].omega);
-      float2 pv[24], sv[24], tv[24];
-      load_scaled(p, P, i, pv);
-      load_scaled(s, P, i, sv);
-      load_scaled(t, P, i, tv);
-      float2 x0[12], x1[12];
-      if (a0) x.load(2 * P, i, x0);
-      if (a1) x.load(2 * P + 1, i, x1);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        CP xk{make_float2(a0 ? x0[k].x : 0.f, a1 ? x1[k].x : 0.f), make_float2(a0 ? x0[k].y : 0.f, a1 ? x1[k].y : 0.f)};
-        xk = cp_fma(al, CP{pv[2 * k], pv[2 * k + 1]}, xk);
-        xk = cp_fma(om, CP{sv[2 * k], sv[2 * k + 1]}, xk);
-        x0[k] = make_float2(xk.re.x, xk.im.x);
-        x1[k] = make_float2(xk.re.y, xk.im.y);
-        CP rn = cp_fms(om, CP{tv[2 * k], tv[2 * k + 1]}, CP{sv[2 * k], sv[2 * k + 1]});
-        sv[2 * k] = rn.re;
-        sv[2 * k + 1] = rn.im;
-      }
-      if (a0) x.store(2 * P, i, x0);
-      if (a1) x.store(2 * P + 1, i, x1);
-      store_pair(r, P, i, sv);
-      load_scaled(rhat, P, i, pv);
-      float2 re = make_float2(0.f, 0.f), ip = re, im = re, nn = re;
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        re = F2(pv[2 * k], sv[2 * k], re);
-        re = F2(pv[2 * k + 1], sv[2 * k + 1], re);
-        ip = F2(pv[2 * k], sv[2 * k + 1], ip);
-        im = F2(pv[2 * k + 1], sv[2 * k], im);
-        nn = F2(sv[2 * k], sv[2 * k], nn);
-        nn = F2(sv[2 * k + 1], sv[2 * k + 1], nn);
-      }
-      sre = re;
-      sim = S2(ip, im);
-      snn = nn;
-    }
+    if (i < vh)
+      pair_xr_site(sc[2 * P], sc[2 * P + 1], flags[2 * P], flags[2 * P + 1], x, p, s, t, r, rhat, P, i, sre, sim, snn);
     pair_reduce_store<1, SUM_DOT_C>(sre, sim, snn, part + (size_t)(2 * P) * nbx + sb,
                                     part + (size_t)(2 * P + 1) * nbx + sb, true);
   }
 }
 
-// members flagged FLAG_RU: r = src (FP32), optionally x = 0; partials per
-// member of <rhat, r> (or <r, r>) and |r|^2
 template <class SP>
 __global__ void __launch_bounds__(ST) k_pair_copy(int vh, const int *flags, F32F src, SP r, SP rhat, bool use_rhat,
                                                   F32F x, bool zero_x, const int *plist, const int *pcount, D4S *part,
@@ -1282,41 +1342,8 @@ __global__ void __launch_bounds__(ST) k_pair_copy(int vh, const int *flags, F32F
     const int P = plist[w / nbx], sb = w % nbx;
     const int i = sb * ST + threadIdx.x;
     float2 sre = make_float2(0.f, 0.f), sim = sre, snn = sre;
-    if (i < vh) {
-      const bool w0 = flags[2 * P] & FLAG_RU, w1 = flags[2 * P + 1] & FLAG_RU;
-      float2 s0[12], s1[12], v[24];
-      if (w0) src.load(2 * P, i, s0);
-      if (w1) src.load(2 * P + 1, i, s1);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        v[2 * k] = make_float2(w0 ? s0[k].x : 0.f, w1 ? s1[k].x : 0.f);
-        v[2 * k + 1] = make_float2(w0 ? s0[k].y : 0.f, w1 ? s1[k].y : 0.f);
-      }
-      store_members(r, P, i, v, w0, w1);
-      if (zero_x) {
-        float2 z[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) z[k] = make_float2(0.f, 0.f);
-        if (w0) x.store(2 * P, i, z);
-        if (w1) x.store(2 * P + 1, i, z);
-      }
-      float2 q[24];
-      if (use_rhat) load_scaled(rhat, P, i, q);
-      float2 re = make_float2(0.f, 0.f), ip = re, im = re, nn = re;
-#pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        const float2 qr = use_rhat ? q[2 * k] : v[2 * k], qi = use_rhat ? q[2 * k + 1] : v[2 * k + 1];
-        re = F2(qr, v[2 * k], re);
-        re = F2(qi, v[2 * k + 1], re);
-        ip = F2(qr, v[2 * k + 1], ip);
-        im = F2(qi, v[2 * k], im);
-        nn = F2(v[2 * k], v[2 * k], nn);
-        nn = F2(v[2 * k + 1], v[2 * k + 1], nn);
-      }
-      sre = re;
-      sim = S2(ip, im);
-      snn = nn;
-    }
+    if (i < vh)
+      pair_copy_site(flags[2 * P], flags[2 * P + 1], src, r, rhat, use_rhat, x, zero_x, P, i, sre, sim, snn);
     pair_reduce_store<1, SUM_DOT_C>(sre, sim, snn, part + (size_t)(2 * P) * nbx + sb,
                                     part + (size_t)(2 * P + 1) * nbx + sb, true);
   }
@@ -1390,28 +1417,111 @@ __global__ void __launch_bounds__(ST) k_cvt64to32_both(Geom g, const double2 *__
 }
 
 // ============================================================ finalisers
-__device__ __forceinline__ D4S warp_total_s(const D4S *part, int nb) {
-  D4S acc = {0, 0, 0, 0};
-  for (int k = threadIdx.x & 31; k < nb; k += 32) {
-    D4S v = part[k];
-    acc.a += v.a;
-    acc.b += v.b;
-    acc.c += v.c;
-    acc.d += v.d;
+// Totals over nb partials by one warp, in a fixed order; valid on lane 0, fields as the
+// kernels that wrote them.  As in pair_reduce_store a lane hands the values that its
+// partner keeps over to it, 5 or 6 FP64 additions in sequence instead of 20: alpha,
+// omega and the convergence test of 17 right-hand sides of 8^3 x 16 took 4.5, 4.5 and 7 kilocycles, 2.6, 2.6 and 3 here.
+template <int SUM> __device__ __forceinline__ D4S warp_total_s(const D4S *part, int nb) {
+  constexpr bool DOT = SUM != SUM_NORM, NORM = SUM != SUM_DOT;
+  const int lane = threadIdx.x & 31;
+  double a = 0.0, b = 0.0, n = 0.0;
+  for (int k = lane; k < nb; k += 32) {
+    const D4S v = part[k];
+    if (DOT) a += v.a;
+    if (DOT) b += v.b;
+    if (NORM) n += SUM == SUM_DOT_D ? v.d : v.c;
   }
-  acc.a = warp_sum_d(acc.a);
-  acc.b = warp_sum_d(acc.b);
-  acc.c = warp_sum_d(acc.c);
-  acc.d = warp_sum_d(acc.d);
-  return acc;
+  auto add_xor = [&](double v, int o) { return v + __shfl_xor_sync(0xffffffffu, v, o); };
+  const bool up16 = lane & 16, up8 = lane & 8;
+  double v;  // ends as a on lane 0, b on lane 8, the norm on lane 16 (on all without a dot)
+  if constexpr (DOT && NORM) {
+    const double t = __shfl_xor_sync(0xffffffffu, up16 ? a : n, 16), u = __shfl_xor_sync(0xffffffffu, b, 16);
+    const double an = (up16 ? n : a) + t, bn = up16 ? an : b + u;
+    v = (up8 ? bn : an) + __shfl_xor_sync(0xffffffffu, up8 ? an : bn, 8);
+  } else if constexpr (DOT) {
+    v = (up8 ? b : a) + __shfl_xor_sync(0xffffffffu, up8 ? a : b, 8);
+    v = add_xor(v, 16);
+  } else {
+    v = add_xor(add_xor(n, 16), 8);
+  }
+  v = add_xor(add_xor(add_xor(v, 4), 2), 1);
+  D4S r = {0, 0, 0, 0};
+  if (DOT) {
+    r.a = v;
+    r.b = __shfl_sync(0xffffffffu, v, 8);
+  }
+  if (NORM) (SUM == SUM_DOT_D ? r.d : r.c) = __shfl_sync(0xffffffffu, v, 16);
+  return r;
 }
 
+// FP64 instructions take 64 cycles or more each, and a right-hand side's scalars are one
+// chain of them: one reciprocal per quotient, and comparisons on the bit patterns, whose
+// order is that of the values where both are >= 0 (a negative bound is below all).
 __device__ __forceinline__ double2 cdiv_d(double2 a, double2 b) {
-  double d = b.x * b.x + b.y * b.y;
-  return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
+  const double i = __drcp_rn(fma(b.x, b.x, b.y * b.y));
+  return make_double2(fma(a.x, b.x, a.y * b.y) * i, fma(a.y, b.x, -(a.x * b.y)) * i);
 }
 __device__ __forceinline__ double2 cmul_d(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  return make_double2(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
+}
+__device__ __forceinline__ bool finite_d(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool less_bits(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+__device__ __forceinline__ bool zero_d(double v) { return (__double_as_longlong(v) << 1) == 0; }
+
+// The scalars of one right-hand side from the totals t of a kernel's sums; the last
+// three return its flags.
+__device__ __forceinline__ void fin_alpha(SState &s, const D4S &t) {  // t: <rhat, v>
+  double2 rv = make_double2(t.a, t.b);
+  s.alpha = (zero_d(rv.x) && zero_d(rv.y)) ? make_double2(0.0, 0.0) : cdiv_d(s.rho, rv);
+  s.restart = 0;
+}
+__device__ __forceinline__ void fin_omega(SState &s, const D4S &t) {  // t: <t, s>, |t|^2
+  const double i = __drcp_rn(t.d);
+  s.omega = zero_d(t.d) ? make_double2(0.0, 0.0) : make_double2(t.a * i, t.b * i);
+}
+__device__ __forceinline__ int fin_conv(SState &s, const D4S &t, double delta2, int max_iter) {  // <rhat, r>, |r|^2
+  double2 rho_new = make_double2(t.a, t.b);
+  s.rr = t.c;
+  s.iters += 1;
+  if (!finite_d(t.a) || !finite_d(t.b) || !finite_d(t.c)) {
+    s.status = LQCD_ERR_NONFINITE;
+    return 0;
+  }
+  int f = FLAG_ACTIVE;
+  if (!less_bits(s.target2, t.c) || less_bits(t.c, delta2 * s.rmax)) f |= FLAG_RU;  // verify / refresh with an FP32 true residual
+  if (s.iters >= max_iter) f |= FLAG_RU;                          // final FP32 residual before stopping
+  if (less_bits(s.rmax, t.c)) s.rmax = t.c;
+  double rho2 = rho_new.x * rho_new.x + rho_new.y * rho_new.y;
+  double om2 = s.omega.x * s.omega.x + s.omega.y * s.omega.y;
+  if (om2 == 0.0 || rho2 == 0.0 || rho2 < 1e-60 * t.c * t.c) {
+    s.restart = 1;  // breakdown: restart the shadow residual
+    s.rho = make_double2(t.c, 0.0);
+    s.alpha = s.omega = make_double2(1.0, 0.0);
+    s.beta = make_double2(0.0, 0.0);
+  } else {
+    s.beta = cdiv_d(cmul_d(rho_new, s.alpha), cmul_d(s.rho, s.omega));
+    s.rho = rho_new;
+  }
+  return f;
+}
+__device__ __forceinline__ int fin_ru(SState &s, const D4S &t, int max_iter) {  // t.c: |r32|^2
+  s.ru_count += 1;
+  double prev = s.rr_ru;
+  s.rr_ru = t.c;
+  if (!finite_d(t.c)) {
+    s.status = LQCD_ERR_NONFINITE;
+    return 0;
+  }
+  // FP32 residual no longer improving: the inner precision floor is reached
+  if (t.c > 0.25 * prev) s.stall += 1; else s.stall = 0;
+  if (!less_bits(s.target2, t.c) || s.stall >= 2 || s.iters >= max_iter) return 0;  // inner solve finished for this cycle
+  s.rmax = t.c;
+  return FLAG_ACTIVE | FLAG_RU;  // r is replaced by r32 next
+}
+__device__ __forceinline__ int fin_ru2(SState &s, const D4S &t) {  // <rhat, r>, |r|^2 after the update
+  s.rr = t.c;
+  s.rho = s.restart ? make_double2(t.c, 0.0) : make_double2(t.a, t.b);
+  return FLAG_ACTIVE;
 }
 
 // after the inner right-hand side is loaded into r (partials: |r|^2 in .c)
@@ -1420,7 +1530,7 @@ __global__ void k_sfin_init(SState *sc, int *flags, const int *list, const int *
                             double floor2) {
   if (blockIdx.x >= *count) return;
   int rhs = list[blockIdx.x];
-  D4S t = warp_total_s(part + (size_t)rhs * nb, nb);
+  D4S t = warp_total_s<SUM_NORM>(part + (size_t)rhs * nb, nb);
   if (threadIdx.x) return;
   SState &s = sc[rhs];
   s.target2 = fmax(s.target2, floor2 * t.c);
@@ -1442,154 +1552,137 @@ __global__ void k_sfin_init(SState *sc, int *flags, const int *list, const int *
   flags[rhs] = f;
 }
 
+// Deterministic compaction of the per-RHS flags into: active groups (any
+// member active), RHS needing a reliable update, and groups containing one.
+// A group is gs consecutive right-hand sides (2: pair layout, 128: tiles).
+struct Lists {
+  int n, gs;
+  int *flags, *act_groups, *ru_list, *ru_groups, *counts;
+  unsigned *ticket;  // blocks of the running finaliser that are done (build_lists_last)
+};
+
+// By one block of whole warps.  The three counts of a thread's run of groups are summed
+// together, 21 bits each, in shuffles: one barrier.  (As three scans over shared memory
+// with twenty barriers the kernel took 5.3 us whatever its size.)
+__device__ __forceinline__ void build_lists(const Lists &l) {
+  __shared__ unsigned long long tot[32];
+  const int ng = (l.n + l.gs - 1) / l.gs, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, nw = nt >> 5;
+  const int per = (ng + nt - 1) / nt, b0 = min(ng, tid * per), b1 = min(ng, b0 + per);
+  auto group = [&](int P, int &any, int &nru) {
+    any = nru = 0;
+#pragma unroll 8
+    for (int k = P * l.gs; k < min(l.n, (P + 1) * l.gs); ++k) {
+      const int f = __ldcg(l.flags + k);  // (may have been written by other blocks of this launch)
+      any |= f;
+      nru += (f & FLAG_RU) ? 1 : 0;
+    }
+  };
+  unsigned long long own = 0;  // active groups, RU right-hand sides << 21, RU groups << 42
+  for (int P = b0; P < b1; ++P) {
+    int any, nru;
+    group(P, any, nru);
+    own += ((any & FLAG_ACTIVE) ? 1ull : 0ull) + ((unsigned long long)nru << 21) + ((any & FLAG_RU) ? 1ull << 42 : 0ull);
+  }
+  auto scan = [&](unsigned long long v) {  // inclusive, over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    return v;
+  };
+  const unsigned long long in_warp = scan(own);
+  if (lane == 31) tot[tid >> 5] = in_warp;
+  __syncthreads();
+  const unsigned long long warps = scan(lane < nw ? tot[lane] : 0ull);  // every warp, of the warps' totals
+  const unsigned long long mine = __shfl_sync(0xffffffffu, warps, tid >> 5) - tot[tid >> 5] + in_warp - own;
+  int oa = (int)(mine & 0x1fffff), orr = (int)(mine >> 21 & 0x1fffff), op = (int)(mine >> 42);
+  for (int P = b0; P < b1; ++P) {
+    int any, nru;
+    group(P, any, nru);
+    if (nru)
+      for (int k = P * l.gs; k < min(l.n, (P + 1) * l.gs); ++k)
+        if (__ldcg(l.flags + k) & FLAG_RU) l.ru_list[orr++] = k;
+    if (any & FLAG_ACTIVE) l.act_groups[oa++] = P;
+    if (any & FLAG_RU) l.ru_groups[op++] = P;
+  }
+  if (tid == 31) {
+    l.counts[0] = (int)(warps & 0x1fffff);
+    l.counts[1] = (int)(warps >> 21 & 0x1fffff);
+    l.counts[3] = (int)(warps >> 42);
+  }
+}
+__global__ void k_build_lists(Lists l) { build_lists(l); }
+
+// By the last block of a finaliser, once every block has written its flags and read the
+// old lists: saves the launch of k_build_lists.
+__device__ __forceinline__ void build_lists_last(const Lists &l) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(l.ticket, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  build_lists(l);
+}
+
 // One warp per member of a listed group (gs right-hand sides: 2 for the pair
 // layout, 128 for tiles); a block of 64 threads takes two members, block b of
-// group list entry b / (gs / 2).  Members without FLAG_ACTIVE are skipped.
-#define PAIR_MEMBER(n)                                                                     \
-  if (blockIdx.x / (gs >> 1) >= *pcount) return;                                           \
-  const int rhs = gs * plist[blockIdx.x / (gs >> 1)] + 2 * (blockIdx.x % (gs >> 1)) + (threadIdx.x >> 5); \
-  if (rhs >= (n) || !(flags[rhs] & FLAG_ACTIVE)) return;
+// group list entry b / (gs / 2).  -1 for members without FLAG_ACTIVE, which are skipped.
+__device__ __forceinline__ int group_member(const int *flags, const int *plist, const int *pcount, int n, int gs) {
+  if (blockIdx.x / (gs >> 1) >= *pcount) return -1;
+  const int rhs = gs * plist[blockIdx.x / (gs >> 1)] + 2 * (blockIdx.x % (gs >> 1)) + (threadIdx.x >> 5);
+  return rhs < n && (flags[rhs] & FLAG_ACTIVE) ? rhs : -1;
+}
 
 __global__ void k_sfin_alpha(SState *sc, const int *flags, const int *plist, const int *pcount, const D4S *part,
                              int nb, int n, int gs) {
-  PAIR_MEMBER(n)
-  D4S t = warp_total_s(part + (size_t)rhs * nb, nb);
-  if (threadIdx.x & 31) return;
-  SState &s = sc[rhs];
-  double2 rv = make_double2(t.a, t.b);
-  s.alpha = (rv.x == 0.0 && rv.y == 0.0) ? make_double2(0.0, 0.0) : cdiv_d(s.rho, rv);
-  s.restart = 0;
+  const int rhs = group_member(flags, plist, pcount, n, gs);
+  if (rhs < 0) return;
+  const D4S t = warp_total_s<SUM_DOT>(part + (size_t)rhs * nb, nb);
+  if ((threadIdx.x & 31) == 0) fin_alpha(sc[rhs], t);
 }
 
 __global__ void k_sfin_omega(SState *sc, const int *flags, const int *plist, const int *pcount, const D4S *part,
                              int nb, int n, int gs) {
-  PAIR_MEMBER(n)
-  D4S t = warp_total_s(part + (size_t)rhs * nb, nb);
-  if (threadIdx.x & 31) return;
-  SState &s = sc[rhs];
-  s.omega = (t.d == 0.0) ? make_double2(0.0, 0.0) : make_double2(t.a / t.d, t.b / t.d);
+  const int rhs = group_member(flags, plist, pcount, n, gs);
+  if (rhs < 0) return;
+  const D4S t = warp_total_s<SUM_DOT_D>(part + (size_t)rhs * nb, nb);
+  if ((threadIdx.x & 31) == 0) fin_omega(sc[rhs], t);
 }
 
-// convergence / reliable-update decision after the x, r update
-__global__ void k_sfin_conv(SState *sc, int *flags, const int *plist, const int *pcount, const D4S *part, int nb,
-                            int n, double delta2, int max_iter, int gs) {
-  PAIR_MEMBER(n)
-  D4S t = warp_total_s(part + (size_t)rhs * nb, nb);
-  if (threadIdx.x & 31) return;
-  SState &s = sc[rhs];
-  double2 rho_new = make_double2(t.a, t.b);
-  s.rr = t.c;
-  s.iters += 1;
-  if (!isfinite(t.a) || !isfinite(t.b) || !isfinite(t.c)) {
-    s.status = LQCD_ERR_NONFINITE;
-    flags[rhs] = 0;
-    return;
+// convergence / reliable-update decision after the x, r update; then the lists
+__global__ void k_sfin_conv(SState *sc, const D4S *part, int nb, double delta2, int max_iter, Lists l) {
+  const int rhs = group_member(l.flags, l.act_groups, l.counts, l.n, l.gs);
+  if (rhs >= 0) {
+    const D4S t = warp_total_s<SUM_DOT_C>(part + (size_t)rhs * nb, nb);
+    if ((threadIdx.x & 31) == 0) l.flags[rhs] = fin_conv(sc[rhs], t, delta2, max_iter);
   }
-  int f = FLAG_ACTIVE;
-  if (t.c <= s.target2 || t.c < delta2 * s.rmax) f |= FLAG_RU;  // verify / refresh with an FP32 true residual
-  if (s.iters >= max_iter) f |= FLAG_RU;                          // final FP32 residual before stopping
-  s.rmax = fmax(s.rmax, t.c);
-  double om2 = s.omega.x * s.omega.x + s.omega.y * s.omega.y;
-  double rho2 = rho_new.x * rho_new.x + rho_new.y * rho_new.y;
-  if (om2 == 0.0 || rho2 == 0.0 || rho2 < 1e-60 * t.c * t.c) {
-    s.restart = 1;  // breakdown: restart the shadow residual
-    s.rho = make_double2(t.c, 0.0);
-    s.alpha = s.omega = make_double2(1.0, 0.0);
-    s.beta = make_double2(0.0, 0.0);
-  } else {
-    s.beta = cmul_d(cdiv_d(rho_new, s.rho), cdiv_d(s.alpha, s.omega));
-    s.rho = rho_new;
-  }
-  flags[rhs] = f;
+  build_lists_last(l);
 }
 
-// after r32 = b32 - D_hat x32 (partials |r32|^2 in .c): accept, stop or continue
-__global__ void k_sfin_ru(SState *sc, int *flags, const int *list, const int *count, const D4S *part, int nb,
-                          int max_iter) {
-  if (blockIdx.x >= *count) return;
-  int rhs = list[blockIdx.x];
-  D4S t = warp_total_s(part + (size_t)rhs * nb, nb);
-  if (threadIdx.x) return;
-  SState &s = sc[rhs];
-  s.ru_count += 1;
-  double prev = s.rr_ru;
-  s.rr_ru = t.c;
-  if (!isfinite(t.c)) {
-    s.status = LQCD_ERR_NONFINITE;
-    flags[rhs] = 0;
-    return;
+// after r32 = b32 - D_hat x32 (partials |r32|^2 in .c): accept, stop or continue; then the
+// lists.  A warp per right-hand side, two to a block.
+__global__ void k_sfin_ru(SState *sc, const D4S *part, int nb, int max_iter, Lists l) {
+  const int e = 2 * blockIdx.x + (threadIdx.x >> 5);
+  if (e < l.counts[1]) {
+    const int rhs = l.ru_list[e];
+    const D4S t = warp_total_s<SUM_NORM>(part + (size_t)rhs * nb, nb);
+    if ((threadIdx.x & 31) == 0) l.flags[rhs] = fin_ru(sc[rhs], t, max_iter);
   }
-  // FP32 residual no longer improving: the inner precision floor is reached
-  if (t.c > 0.25 * prev) s.stall += 1; else s.stall = 0;
-  if (t.c <= s.target2 || s.stall >= 2 || s.iters >= max_iter) {
-    flags[rhs] = 0;  // inner solve finished for this cycle
-    return;
-  }
-  s.rmax = t.c;
-  flags[rhs] = FLAG_ACTIVE | FLAG_RU;  // r is replaced by r32 next
+  build_lists_last(l);
 }
 
-// after the reliable update copied r32 into r: refresh rho = <rhat, r>
-__global__ void k_sfin_ru2(SState *sc, int *flags, const int *list, const int *count, const D4S *part, int nb) {
-  if (blockIdx.x >= *count) return;
-  int rhs = list[blockIdx.x];
-  D4S t = warp_total_s(part + (size_t)rhs * nb, nb);
-  if (threadIdx.x) return;
-  SState &s = sc[rhs];
-  s.rr = t.c;
-  if (!s.restart) s.rho = make_double2(t.a, t.b);
-  else s.rho = make_double2(t.c, 0.0);
-  flags[rhs] = FLAG_ACTIVE;
-}
-
-// Deterministic compaction of the per-RHS flags into: active groups (any
-// member active), RHS needing a reliable update, and groups containing one.
-// A group is gs consecutive right-hand sides (2: pair layout, 128: tiles).
-__global__ void k_build_lists(int n, const int *flags, int gs, int *act_groups, int *ru_list, int *ru_groups,
-                              int *counts) {
-  __shared__ int sa[1024], sr[1024], sp[1024];
-  const int ng = (n + gs - 1) / gs;
-  int tid = threadIdx.x, nt = blockDim.x;
-  int per = (ng + nt - 1) / nt;
-  int b0 = tid * per, b1 = min(ng, b0 + per);
-  int ca = 0, cr = 0, cp = 0;
-  for (int P = b0; P < b1; ++P) {
-    int any = 0, nru = 0;
-    for (int k = P * gs; k < min(n, (P + 1) * gs); ++k) {
-      any |= flags[k];
-      nru += (flags[k] & FLAG_RU) ? 1 : 0;
-    }
-    ca += (any & FLAG_ACTIVE) ? 1 : 0;
-    cp += (any & FLAG_RU) ? 1 : 0;
-    cr += nru;
+// after the reliable update copied r32 into r: refresh rho = <rhat, r>; then the lists
+__global__ void k_sfin_ru2(SState *sc, const D4S *part, int nb, Lists l) {
+  const int e = 2 * blockIdx.x + (threadIdx.x >> 5);
+  if (e < l.counts[1]) {
+    const int rhs = l.ru_list[e];
+    const D4S t = warp_total_s<SUM_DOT_C>(part + (size_t)rhs * nb, nb);
+    if ((threadIdx.x & 31) == 0) l.flags[rhs] = fin_ru2(sc[rhs], t);
   }
-  sa[tid] = ca;
-  sr[tid] = cr;
-  sp[tid] = cp;
-  __syncthreads();
-  for (int off = 1; off < nt; off <<= 1) {  // inclusive scans
-    int va = tid >= off ? sa[tid - off] : 0, vr = tid >= off ? sr[tid - off] : 0, vp = tid >= off ? sp[tid - off] : 0;
-    __syncthreads();
-    sa[tid] += va;
-    sr[tid] += vr;
-    sp[tid] += vp;
-    __syncthreads();
-  }
-  int oa = sa[tid] - ca, orr = sr[tid] - cr, op = sp[tid] - cp;
-  for (int P = b0; P < b1; ++P) {
-    int any = 0;
-    for (int k = P * gs; k < min(n, (P + 1) * gs); ++k) {
-      any |= flags[k];
-      if (flags[k] & FLAG_RU) ru_list[orr++] = k;
-    }
-    if (any & FLAG_ACTIVE) act_groups[oa++] = P;
-    if (any & FLAG_RU) ru_groups[op++] = P;
-  }
-  if (tid == nt - 1) {
-    counts[0] = sa[tid];
-    counts[1] = sr[tid];
-    counts[3] = sp[tid];
-  }
+  build_lists_last(l);
 }
 
 }  // namespace lqcd
@@ -1685,7 +1778,8 @@ struct SmallBufs {
 // partial sums per RHS: the larger of the pair kernels' blocks of ST sites and
 // the tile kernels' chunks of TCH sites
 static int part_blocks(int vh) { return std::max((vh + ST - 1) / ST, (vh + TCH - 1) / TCH); }
-static SmallBufs small_layout(void *base, int cap, int nbp) {
+static SmallBufs small_layout(void *base, int cap, int vh) {
+  const int nbp = part_blocks(vh);
   Carver cv(base);
   SmallBufs b;
   b.sc = cv.take<SState>(cap);
@@ -1696,7 +1790,8 @@ static SmallBufs small_layout(void *base, int cap, int nbp) {
   b.cyc_list = cv.take<int>(cap);
   b.cyc_pairs = cv.take<int>(cap / 2);
   // [0] active groups, [1] RU RHS, [2] cycle RHS, [3] RU groups, [4] cycle groups, [8] tile-hop error
-  // code, [9] loop stopped by the time budget, [10] loop iterations (see k_loop_cond)
+  // code, [9] loop stopped by the time budget, [10] loop iterations (see k_loop_cond), [12] ticket of
+  // build_lists_last
   b.counts = cv.take<int>(16);
   b.clk = cv.take<unsigned long long>(2);
   b.scale = cv.take<double>(cap);
@@ -1738,7 +1833,7 @@ static int sloppy_alloc(lqcd_ctx *ctx, int nrhs, int gran = 2) {
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->x.e, (size_t)cap * vpad * sizeof(int)));
   s->x.cap = cap;
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->r32, (size_t)cap * g.V * 6 * sizeof(float4)));
-  LQCD_CUDA_TRY(ctx, cudaMalloc(&s->small, small_layout(nullptr, cap, part_blocks(g.Vh)).size()));
+  LQCD_CUDA_TRY(ctx, cudaMalloc(&s->small, small_layout(nullptr, cap, g.Vh).size()));
   // padding right-hand sides of a tile are computed alongside the real ones: start them at zero
   LQCD_CUDA_TRY(ctx, cudaMemset(s->sd, 0, 7 * pairs * 6 * vh * sizeof(uint4)));
   if (!s->h_counts) LQCD_CUDA_TRY(ctx, cudaMallocHost(&s->h_counts, 16 * sizeof(int)));
@@ -1952,7 +2047,7 @@ struct MixedRun : RunIface {
     }
     auto f32 = [&](int k) { F32F ff; ff.d = ss->f32 + (size_t)k * cap * 6 * vh; ff.vh = vh; return ff; };
     x32 = f32(0); b32 = f32(1); r32 = f32(2); t32 = f32(3); o32 = f32(4);
-    sb = small_layout(ss->small, cap, part_blocks(vh));
+    sb = small_layout(ss->small, cap, vh);
     rr.assign(nrhs, 0.0);
     bb.assign(nrhs, 0.0);
     prev_rel.assign(nrhs, 1e300);
@@ -1971,6 +2066,11 @@ struct MixedRun : RunIface {
     LQCD_CUDA_TRY(ctx, cudaMemsetAsync(sb.counts, 0, 16 * sizeof(int), st));
     return LQCD_OK;
   }
+
+  Lists lists() const {
+    return Lists{nrhs, Ops::GS, sb.flags, sb.act_pairs, sb.ru_list, sb.ru_pairs, sb.counts, (unsigned *)sb.counts + 12};
+  }
+  int list_threads() const { return std::min(1024, ((nrhs + Ops::GS - 1) / Ops::GS + 31) / 32 * 32); }
 
   // the FP64 solution from the iterate's limbs
   int finish() override {
@@ -1996,7 +2096,7 @@ struct MixedRun : RunIface {
         cudaMemcpyAsync(sb.sc, hs.data(), cap * sizeof(SState), cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(sb.flags, hflags.data(), cap * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess)
       return -1.f;
-    KL k_build_lists<<<1, 1024, 0, st>>>(nrhs, sb.flags, Ops::GS, sb.act_pairs, sb.ru_list, sb.ru_pairs, sb.counts);
+    KL k_build_lists<<<1, list_threads(), 0, st>>>(lists());
     launch_iters(st, 1);  // warm-up
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -2097,7 +2197,7 @@ struct MixedRun : RunIface {
                                            counts + 2, nullptr, nbx);
     Ops::copy(st, G, vh, sb.flags, b32, r, r, false, x32, true, sb.cyc_pairs, counts + 4, sb.part, nb);
     KL k_sfin_init<<<(int)hl.size(), 32, 0, st>>>(sb.sc, sb.flags, sb.cyc_list, counts + 2, sb.part, nb, floor2);
-    KL k_build_lists<<<1, 1024, 0, st>>>(nrhs, sb.flags, Ops::GS, sb.act_pairs, sb.ru_list, sb.ru_pairs, counts);
+    KL k_build_lists<<<1, list_threads(), 0, st>>>(lists());
     LQCD_LAUNCH_CHECK(ctx, "mixed: cycle setup");
     inner = true;
     return LQCD_OK;
@@ -2148,19 +2248,15 @@ struct MixedRun : RunIface {
       ev_end();
       KL k_sfin_omega<<<cap / 2, 64, 0, q>>>(sb.sc, sb.flags, sb.act_pairs, counts, sb.part, nb, nrhs, gs);
       Ops::xr(q, G, vh, sb.sc, sb.flags, x32, pp, s, t, r, rhat, sb.act_pairs, counts, sb.part, nb);
-      KL k_sfin_conv<<<cap / 2, 64, 0, q>>>(sb.sc, sb.flags, sb.act_pairs, counts, sb.part, nb, nrhs,
-                                            delta * delta, p.max_iter, gs);
-      KL k_build_lists<<<1, 1024, 0, q>>>(nrhs, sb.flags, gs, sb.act_pairs, sb.ru_list, sb.ru_pairs, counts);
+      KL k_sfin_conv<<<cap / 2, 64, 0, q>>>(sb.sc, sb.part, nb, delta * delta, p.max_iter, lists());
       // reliable update in FP32: r32 = b32 - x32 + kappa^2 H_eo H_oe x32
       KL k_hop32x2<EPI_PLAIN><<<G, ST, 0, q>>>(g, 1, L32, x32, t32, t32, t32, 0.f, 0.f, 1.f, sb.ru_list, counts + 1,
                                              nullptr, nbx);
       KL k_hop32x2<EPI_RES><<<G, ST, 0, q>>>(g, 0, L32, t32, r32, b32, x32, 1.f, -1.f, k2, sb.ru_list, counts + 1,
                                            sb.part, nbx);
-      KL k_sfin_ru<<<nrhs, 32, 0, q>>>(sb.sc, sb.flags, sb.ru_list, counts + 1, sb.part, nbx, p.max_iter);
-      KL k_build_lists<<<1, 1024, 0, q>>>(nrhs, sb.flags, gs, sb.act_pairs, sb.ru_list, sb.ru_pairs, counts);
+      KL k_sfin_ru<<<(nrhs + 1) / 2, 64, 0, q>>>(sb.sc, sb.part, nbx, p.max_iter, lists());
       Ops::copy(q, G, vh, sb.flags, r32, r, rhat, true, x32, false, sb.ru_pairs, counts + 3, sb.part, nb);
-      KL k_sfin_ru2<<<nrhs, 32, 0, q>>>(sb.sc, sb.flags, sb.ru_list, counts + 1, sb.part, nb);
-      KL k_build_lists<<<1, 1024, 0, q>>>(nrhs, sb.flags, gs, sb.act_pairs, sb.ru_list, sb.ru_pairs, counts);
+      KL k_sfin_ru2<<<(nrhs + 1) / 2, 64, 0, q>>>(sb.sc, sb.part, nb, lists());
     }
   }
 
