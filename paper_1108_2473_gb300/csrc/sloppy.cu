@@ -122,11 +122,24 @@ __device__ __forceinline__ void load_raw(const BF16P &f, int P, int i, float2 v[
   }
   nrm = make_float2(1.f, 1.f);
 }
+// a * b that the compiler may not fuse into a following sum: whether it does depends on the
+// kernel around it, and two kernels have to give the same bits (k_pair_solve)
+__device__ __forceinline__ float2 mul2_alone(float2 a, float2 b) {
+  float2 r;
+  asm("{.reg .b64 a, b;\n"
+      " mov.b64 a, {%2, %3};\n"
+      " mov.b64 b, {%4, %5};\n"
+      " mul.rn.f32x2 a, a, b;\n"
+      " mov.b64 {%0, %1}, a;}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
 __device__ __forceinline__ void load_scaled(const F16P &f, int P, int i, float2 v[24]) {
   float2 nrm;
   load_raw(f, P, i, v, nrm);
 #pragma unroll
-  for (int k = 0; k < 24; ++k) v[k] = M2(v[k], nrm);
+  for (int k = 0; k < 24; ++k) v[k] = mul2_alone(v[k], nrm);
 }
 __device__ __forceinline__ void load_scaled(const BF16P &f, int P, int i, float2 v[24]) {
   float2 nrm;
@@ -333,13 +346,26 @@ __device__ __forceinline__ void pair_reduce_store(float2 re, float2 im, float2 n
 }
 
 // One site of the FP32 hopping term for right-hand sides rhs[0], rhs[1]: out = cA A +
-// cB B + cH acc, acc = H in.  EPI_PLAIN: A, B unused.  EPI_AXPY: B unused.  EPI_RES: returns
+// cB B + cH (H in).  EPI_PLAIN: A, B unused.  EPI_AXPY: B unused.  EPI_RES: returns
 // |out|^2 of each.  two: false if rhs[1] only repeats rhs[0], and is not stored.
 template <int EPI>
-__device__ __forceinline__ float2 hop32x2_store(const float2 acc[2][4][3], int i, const F32F &out, const F32F &A,
-                                                const F32F &B, float cA, float cB, float cH, const int rhs[2],
-                                                bool two) {
+__device__ __forceinline__ float2 hop32x2_site(const Geom &g, int p_out, int i, const float4 *links, const F32F &in,
+                                               const F32F &out, const F32F &A, const F32F &B, float cA, float cB,
+                                               float cH, const int rhs[2], bool two) {
   float2 red = make_float2(0.f, 0.f);
+  int c[4];
+  coords_of(g, p_out, i, c);
+  float2 acc[2][4][3];
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) acc[r][a][b] = make_float2(0.f, 0.f);
+  hop_dir32n<0, 2>(g, p_out, c, i, in, rhs, links, acc);
+  hop_dir32n<1, 2>(g, p_out, c, i, in, rhs, links, acc);
+  hop_dir32n<2, 2>(g, p_out, c, i, in, rhs, links, acc);
+  hop_dir32n<3, 2>(g, p_out, c, i, in, rhs, links, acc);
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     float2 o[12];
@@ -384,18 +410,7 @@ __global__ void __launch_bounds__(ST, 4) k_hop32x2(Geom g, int p_out, const floa
     const int rhs[2] = {list[j], two ? list[j + 1] : list[j]};
     const int i = sb * ST + threadIdx.x;
     float2 red = make_float2(0.f, 0.f);  // |out|^2 of the two right-hand sides
-    if (i < g.Vh) {
-      int c[4];
-      coords_of(g, p_out, i, c);
-      float2 acc[2][4][3];
-#pragma unroll
-      for (int k = 0; k < 24; ++k) acc[k / 12][k / 3 % 4][k % 3] = make_float2(0.f, 0.f);
-      hop_dir32n<0, 2>(g, p_out, c, i, in, rhs, links, acc);
-      hop_dir32n<1, 2>(g, p_out, c, i, in, rhs, links, acc);
-      hop_dir32n<2, 2>(g, p_out, c, i, in, rhs, links, acc);
-      hop_dir32n<3, 2>(g, p_out, c, i, in, rhs, links, acc);
-      red = hop32x2_store<EPI>(acc, i, out, A, B, cA, cB, cH, rhs, two);
-    }
+    if (i < g.Vh) red = hop32x2_site<EPI>(g, p_out, i, links, in, out, A, B, cA, cB, cH, rhs, two);
     if (EPI == EPI_RES)  // an odd last entry has only one right-hand side (its second sum is not stored)
       pair_reduce_store<1, SUM_NORM>(red, red, red, part + (size_t)rhs[0] * nbx + sb,
                                      part + (size_t)rhs[1] * nbx + sb, true);
@@ -576,6 +591,21 @@ __device__ __forceinline__ void hop_dir_pair(const Geom &g, int p_out, const int
   }
 }
 
+template <class SP, bool R12 = false>
+__device__ __forceinline__ void hop_pair_site(const Geom &g, int p_out, int i, const uint4 *links, const SP &in, int P,
+                                              CP acc[4][3]) {
+  int c[4];
+  coords_of(g, p_out, i, c);
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) acc[a][b] = CP{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  hop_dir_pair<0, SP, R12>(g, p_out, c, i, in, P, links, acc);
+  hop_dir_pair<1, SP, R12>(g, p_out, c, i, in, P, links, acc);
+  hop_dir_pair<2, SP, R12>(g, p_out, c, i, in, P, links, acc);
+  hop_dir_pair<3, SP, R12>(g, p_out, c, i, in, P, links, acc);
+}
+
 // Epilogue of the pair hopping term at output site i of pair P: o = cH acc
 // (+ cA a unless EPI_PLAIN), stored to out; EPI_DOTR: this site's terms of <B, o> per
 // member; EPI_TS: terms of <o, a> and |o|^2 per member (untouched for EPI_PLAIN).
@@ -647,17 +677,8 @@ __global__ void __launch_bounds__(ST * PPB, MINB) k_hop_pair(Geom g, int p_out, 
       atomicAdd(prof + EPI, (unsigned long long)min(ST, g.Vh - sb * ST) * (2 * P + 1 < nrhs ? 2 : 1));
     float2 sre = make_float2(0.f, 0.f), sim = sre, snn = sre;
     if (valid && i < g.Vh) {
-      int c[4];
-      coords_of(g, p_out, i, c);
       CP acc[4][3];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) acc[a][b] = CP{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      hop_dir_pair<0, SP, R12>(g, p_out, c, i, in, P, links, acc);
-      hop_dir_pair<1, SP, R12>(g, p_out, c, i, in, P, links, acc);
-      hop_dir_pair<2, SP, R12>(g, p_out, c, i, in, P, links, acc);
-      hop_dir_pair<3, SP, R12>(g, p_out, c, i, in, P, links, acc);
+      hop_pair_site<SP, R12>(g, p_out, i, links, in, P, acc);
       float2 a[24];
       if (EPI != EPI_PLAIN) load_scaled(A, P, i, a);
       pair_epilogue<SP, EPI>(acc, a, cA2, cH2, out, B, P, i, sre, sim, snn);
@@ -1164,7 +1185,7 @@ __device__ __forceinline__ CP cp_fms(const CP &s, const CP &z, const CP &a) {  /
 }
 
 // One site of the solver's vector updates for pair P, whose members' scalars are s0, s1
-// and flags f0, f1.
+// and flags f0, f1: shared by the kernels below and k_pair_solve.
 // p = r + beta (p - omega v); members flagged for restart take rhat = r, p = r.
 template <class SP>
 __device__ __forceinline__ void pair_p_site(const SState &s0, const SState &s1, const SP &r, const SP &rhat,
@@ -1419,8 +1440,10 @@ __global__ void __launch_bounds__(ST) k_cvt64to32_both(Geom g, const double2 *__
 // ============================================================ finalisers
 // Totals over nb partials by one warp, in a fixed order; valid on lane 0, fields as the
 // kernels that wrote them.  As in pair_reduce_store a lane hands the values that its
-// partner keeps over to it, 5 or 6 FP64 additions in sequence instead of 20: alpha,
-// omega and the convergence test of 17 right-hand sides of 8^3 x 16 took 4.5, 4.5 and 7 kilocycles, 2.6, 2.6 and 3 here.
+// partner keeps over to it, 5 or 6 FP64 additions in sequence instead of 20.  With the
+// quotients below, alpha and omega of a pair on 8^3 x 16 take 3.7 kilocycles each instead
+// of 6.2.  With the lists built by the finalisers (build_lists_last) a BF16 solve of 12
+// right-hand sides of 4^4 takes 1.09 ms instead of 1.21, 17 of 8^3 x 16 1.47 instead of 1.55.
 template <int SUM> __device__ __forceinline__ D4S warp_total_s(const D4S *part, int nb) {
   constexpr bool DOT = SUM != SUM_NORM, NORM = SUM != SUM_DOT;
   const int lane = threadIdx.x & 31;
@@ -1717,6 +1740,151 @@ __global__ void k_loop_cond(cudaGraphConditionalHandle h, int *counts, const uns
 
 }  // namespace lqcd
 
+// ================================= whole inner solve of a pair in one cluster
+namespace lqcd {
+
+template <int S> using Sum = std::integral_constant<int, S>;
+template <class SP> struct PairSolve {
+  const uint4 *links16;
+  const float4 *links32;
+  SP r, rhat, p, v, s, t, tmp;
+  F32F x32, b32, r32, t32;
+  SState *sc;
+  int *flags, *counts, *late;
+  const int *plist;
+  D4S *part[2];  // two sets of partial sums, used in turn
+  const unsigned long long *clk;
+  int nbx, max_iter, max_loops;
+  float k2, one;  // one: 1, but no constant: what the compiler folds and fuses has to be as in the launched kernels
+  double delta2;
+};
+
+__global__ void k_clock_start(int *counts, unsigned long long *clk) {
+  clk[0] = globaltimer_ns();
+  counts[9] = counts[10] = 0;
+}
+
+// The inner BiCGstab of one pair of right-hand sides per cluster, to the end: the steps
+// of launch_iters, term for term and sum for sum, with a cluster barrier where its
+// kernels end, so the results are those of the launches bit for bit.  Pairs do not depend
+// on each other, so nothing wider is needed.  On a small lattice the launches take 2 us or
+// more each whatever they do (16 to an iteration); here a step costs the latency of its
+// loads and a barrier.  A block takes one block of ST sites, with the registers that two
+// blocks per SM leave (at 128 a thread it spilled).
+// Every block of a cluster sums the partials itself, in one order, and so takes the
+// same decisions: all blocks meet at every barrier.  The two sets of partials alternate:
+// a set is written again only after a barrier that follows its reading.
+template <class SP> __global__ void __launch_bounds__(ST, 2) k_pair_solve(Geom g, PairSolve<SP> a, int cluster) {
+  const int rank = blockIdx.x % cluster, item = blockIdx.x / cluster;
+  if (item >= a.counts[0]) return;  // the whole cluster
+  const int P = a.plist[item], tid = threadIdx.x, i = rank * ST + tid;
+  const bool valid = i < g.Vh;
+  __shared__ SState sc[2];
+  __shared__ int fl[2];
+  auto sync = [&]() {
+    if (cluster == 1) {
+      __syncthreads();
+    } else {
+      asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    }
+  };
+  // this block's partial sums of right-hand sides r0 and r1
+  auto put = [&](auto sum, D4S *part, int r0, int r1, float2 re, float2 im, float2 nn) {
+    pair_reduce_store<1, decltype(sum)::value>(re, im, nn, part + (size_t)r0 * a.nbx + rank,
+                                               part + (size_t)r1 * a.nbx + rank, rank < a.nbx);
+  };
+  // the totals of both members, one warp each; f(member, totals) on its first lane
+  auto finish = [&](auto sum, const D4S *part, int need, auto f) {
+    const int m = tid >> 5;
+    if (m < 2 && (fl[m] & need)) {
+      const D4S t = warp_total_s<decltype(sum)::value>(part + (size_t)(2 * P + m) * a.nbx, a.nbx);
+      if ((tid & 31) == 0) f(m, t);
+    }
+    __syncthreads();
+  };
+  const float2 zero = make_float2(0.f, 0.f);
+  if (tid < 2) {
+    sc[tid] = a.sc[2 * P + tid];
+    fl[tid] = a.flags[2 * P + tid];
+  }
+  __syncthreads();
+  bool late = false;
+  for (int it = 0; it < a.max_loops; ++it) {
+    if (rank == 0 && tid == 0) a.late[P] = globaltimer_ns() - a.clk[0] > a.clk[1] || a.clk[1] == 0;
+    float2 sre, sim, snn;
+#pragma unroll 1
+    for (int h = 0; h < 4; ++h) {  // one loop body: the code stays in the instruction cache
+      if (!(h & 1)) {
+        if (valid) {
+          if (h == 0) pair_p_site(sc[0], sc[1], a.r, a.rhat, a.p, a.v, P, i);
+          else pair_s_site(sc[0], sc[1], a.r, a.v, a.s, P, i);
+        }
+        sync();
+        if (h == 0) {
+          late = *(volatile int *)(a.late + P) != 0;
+          if (late) break;
+        }
+      }
+      sre = sim = snn = zero;
+      if (valid) {
+        CP acc[4][3];
+        hop_pair_site(g, ~h & 1, i, a.links16, h & 1 ? a.tmp : (h == 0 ? a.p : a.s), P, acc);
+        const float2 one = make_float2(a.one, a.one), mk2 = make_float2(-a.k2, -a.k2);
+        float2 A[24];
+        if (h == 1) {
+          load_scaled(a.p, P, i, A);
+          pair_epilogue<SP, EPI_DOTR>(acc, A, one, mk2, a.v, a.rhat, P, i, sre, sim, snn);
+        } else if (h == 3) {
+          load_scaled(a.s, P, i, A);
+          pair_epilogue<SP, EPI_TS>(acc, A, one, mk2, a.t, a.rhat, P, i, sre, sim, snn);
+        } else {
+          pair_epilogue<SP, EPI_PLAIN>(acc, A, one, one, a.tmp, a.rhat, P, i, sre, sim, snn);
+        }
+      }
+      if (h == 1) put(Sum<SUM_DOT>(), a.part[0], 2 * P, 2 * P + 1, sre, sim, snn);
+      if (h == 3) put(Sum<SUM_DOT_D>(), a.part[1], 2 * P, 2 * P + 1, sre, sim, snn);
+      sync();
+      if (h == 1) finish(Sum<SUM_DOT>(), a.part[0], FLAG_ACTIVE, [&](int m, const D4S &t) { fin_alpha(sc[m], t); });
+      if (h == 3) finish(Sum<SUM_DOT_D>(), a.part[1], FLAG_ACTIVE, [&](int m, const D4S &t) { fin_omega(sc[m], t); });
+    }
+    if (late) break;
+    sre = sim = snn = zero;
+    if (valid) pair_xr_site(sc[0], sc[1], fl[0], fl[1], a.x32, a.p, a.s, a.t, a.r, a.rhat, P, i, sre, sim, snn);
+    put(Sum<SUM_DOT_C>(), a.part[0], 2 * P, 2 * P + 1, sre, sim, snn);
+    sync();
+    finish(Sum<SUM_DOT_C>(), a.part[0], FLAG_ACTIVE,
+           [&](int m, const D4S &t) { fl[m] = fin_conv(sc[m], t, a.delta2, a.max_iter); });
+    if ((fl[0] | fl[1]) & FLAG_RU) {  // reliable update in FP32 of the flagged members
+      const bool two = (fl[0] & fl[1]) & FLAG_RU;
+      const int rhs[2] = {fl[0] & FLAG_RU ? 2 * P : 2 * P + 1, fl[1] & FLAG_RU ? 2 * P + 1 : 2 * P};
+      if (valid) hop32x2_site<EPI_PLAIN>(g, 1, i, a.links32, a.x32, a.t32, a.t32, a.t32, 0.f, 0.f, a.one, rhs, two);
+      sync();
+      float2 red = zero;
+      if (valid)
+        red = hop32x2_site<EPI_RES>(g, 0, i, a.links32, a.t32, a.r32, a.b32, a.x32, a.one, -a.one, a.k2, rhs, two);
+      put(Sum<SUM_NORM>(), a.part[1], rhs[0], rhs[1], red, red, red);
+      sync();
+      finish(Sum<SUM_NORM>(), a.part[1], FLAG_RU, [&](int m, const D4S &t) { fl[m] = fin_ru(sc[m], t, a.max_iter); });
+      if ((fl[0] | fl[1]) & FLAG_RU) {
+        sre = sim = snn = zero;
+        if (valid) pair_copy_site(fl[0], fl[1], a.r32, a.r, a.rhat, true, a.x32, false, P, i, sre, sim, snn);
+        put(Sum<SUM_DOT_C>(), a.part[0], 2 * P, 2 * P + 1, sre, sim, snn);
+        sync();
+        finish(Sum<SUM_DOT_C>(), a.part[0], FLAG_RU, [&](int m, const D4S &t) { fl[m] = fin_ru2(sc[m], t); });
+      }
+    }
+    if (!((fl[0] | fl[1]) & FLAG_ACTIVE)) break;
+  }
+  if (rank == 0 && tid < 2) {
+    a.sc[2 * P + tid] = sc[tid];
+    a.flags[2 * P + tid] = fl[tid];
+    if (late) a.counts[9] = 1;
+  }
+}
+
+}  // namespace lqcd
+
 // ======================================================== host-side driver
 namespace lqcd {
 
@@ -1770,7 +1938,8 @@ struct SmallBufs {
   SState *sc;
   int *flags, *act_pairs, *ru_list, *ru_pairs, *cyc_list, *cyc_pairs, *counts;
   double *scale, *unscale;
-  D4S *part;
+  D4S *part, *part2;  // part2: second set for k_pair_solve
+  int *late;
   unsigned long long *clk;  // loop start and budget (ns)
   size_t bytes;
   size_t size() const { return bytes; }
@@ -1778,8 +1947,10 @@ struct SmallBufs {
 // partial sums per RHS: the larger of the pair kernels' blocks of ST sites and
 // the tile kernels' chunks of TCH sites
 static int part_blocks(int vh) { return std::max((vh + ST - 1) / ST, (vh + TCH - 1) / TCH); }
+// blocks of ST sites up to which a solve may take one cluster per pair (k_pair_solve)
+constexpr int SOLO_NBX = 16;
 static SmallBufs small_layout(void *base, int cap, int vh) {
-  const int nbp = part_blocks(vh);
+  const int nbp = part_blocks(vh), nbx = (vh + ST - 1) / ST;
   Carver cv(base);
   SmallBufs b;
   b.sc = cv.take<SState>(cap);
@@ -1797,6 +1968,8 @@ static SmallBufs small_layout(void *base, int cap, int vh) {
   b.scale = cv.take<double>(cap);
   b.unscale = cv.take<double>(cap);
   b.part = cv.take<D4S>((size_t)cap * nbp);
+  b.part2 = cv.take<D4S>(nbx <= SOLO_NBX ? (size_t)cap * nbx : 0);
+  b.late = cv.take<int>(cap / 2);
   b.bytes = cv.size();
   return b;
 }
@@ -1975,6 +2148,8 @@ struct RunIface {
   virtual int init() = 0;
   virtual int cycle_start() = 0;
   virtual void launch_iters(cudaStream_t q, int k) = 0;
+  virtual bool solo() const = 0;  // the inner solve is one kernel (launch_solo)
+  virtual cudaError_t launch_solo(cudaStream_t q) = 0;
   virtual int request_count(cudaStream_t q) = 0;
   virtual int poll() = 0;
   virtual int finish() = 0;
@@ -2260,6 +2435,51 @@ struct MixedRun : RunIface {
     }
   }
 
+  // One cluster per pair of right-hand sides (k_pair_solve) where nearly all clusters run
+  // at once (two blocks fit an SM): there the latency of the launches is what bounds a
+  // solve.  BF16: 12 right-hand sides of 4^4 1.19 -> 0.83 ms, 12 / 24 of 8^4 1.23 -> 0.96
+  // and 1.43 -> 1.14, 60 of 6^4 1.44 -> 1.11; with more the launches' wider grids win (38
+  // and 96 of 8^4: 1.60 and 2.62 ms against 1.68 and 3.05 here, 96 of 6^4 1.56 against
+  // 1.62).  The switches that name the other path's launches keep it.
+  bool solo() const override {
+    if (Ops::GS != 2 || nbx > SOLO_NBX || ctx->prof_on || force_code >= 0) return false;
+    if (getenv("LQCD_NO_GRAPH") || getenv("LQCD_HOP_VARIANT")) return false;
+    return 3ll * npairs * solo_cluster() <= 4ll * num_sms(ctx->device);
+  }
+  int solo_cluster() const {
+    int c = 1;
+    while (c < nbx) c *= 2;
+    return c;
+  }
+  cudaError_t launch_solo(cudaStream_t q) override {
+    if constexpr (Ops::GS != 2) {
+      return cudaErrorNotSupported;
+    } else {
+      PairSolve<SF> a{ctx->U16, ctx->U32, r, rhat, pp, v, s, t, tmp, x32, b32, r32, t32, sb.sc, sb.flags, sb.counts, sb.late,
+                      sb.act_pairs, {sb.part, sb.part2}, sb.clk, nbx, p.max_iter, p.max_iter + 1, k2, 1.f, delta * delta};
+      KL k_clock_start<<<1, 1, 0, q>>>(sb.counts, sb.clk);
+      const int C = solo_cluster();
+      auto kern = k_pair_solve<SF>;
+      cudaError_t e = cudaSuccess;
+      if (C > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(npairs * C);
+      cfg.blockDim = dim3(ST);
+      cfg.stream = q;
+      cudaLaunchAttribute at = {};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = C;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      e = (KL cudaLaunchKernelEx(&cfg, kern, g, a, C));
+      if (e != cudaSuccess) return e;
+      KL k_build_lists<<<1, list_threads(), 0, q>>>(lists());
+      return cudaGetLastError();
+    }
+  }
+
   // enqueue the read-back of the active count, the tile hop's error code and
   // the device loop's budget flag and iteration count
   int request_count(cudaStream_t q) override {
@@ -2421,7 +2641,8 @@ static int mixed_block(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, co
   // iterations directly: recording a graph takes longer than it saves once, and a
   // program that solves once on the default stream does not pay for it.  12 point
   // sources of 4^4: 1.70 -> 1.20 ms, 17 sources of 8^3 x 16 (FP16): 2.94 -> 2.00 ms.
-  bool use_graph = !ctx->prof_on && getenv("LQCD_NO_GRAPH") == nullptr;
+  bool solo = run->solo();
+  bool use_graph = !solo && !ctx->prof_on && getenv("LQCD_NO_GRAPH") == nullptr;
   if (use_graph && (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread)) {
     const std::vector<double> key = run->graph_key();
     const bool have = ss->graph && ss->graph_key == key;
@@ -2457,7 +2678,11 @@ static int mixed_block(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, co
       }
       run->loop_kernels = ss->graph_kernels;
       LQCD_CUDA_TRY(ctx, cudaGraphLaunch(ss->graph, st));
-    } else {
+    } else if (solo && run->launch_solo(st) != cudaSuccess) {
+      cudaGetLastError();  // clusters of that size refused: launched step by step
+      solo = false;
+      continue;
+    } else if (!solo) {
       run->launch_iters(st, ITERS_PER_POLL);
       LQCD_LAUNCH_CHECK(ctx, "mixed: iteration");
     }
