@@ -1898,6 +1898,7 @@ struct SloppyState {
   float4 *r32 = nullptr;   // residual b - D x, FP32 [2 parity][cap][6][Vh] (seeds the next inner solve)
   char *small = nullptr;
   int *h_counts = nullptr;  // pinned
+  char *h_small = nullptr;  // pinned: the head of `small`
   // captured graph of the inner loop, valid while graph_key matches
   cudaGraphExec_t graph = nullptr;
   std::vector<double> graph_key;
@@ -1917,6 +1918,7 @@ void sloppy_free(lqcd_ctx *ctx) {
   cudaFree(s->r32);
   cudaFree(s->small);
   if (s->h_counts) cudaFreeHost(s->h_counts);
+  if (s->h_small) cudaFreeHost(s->h_small);
   if (s->graph) cudaGraphExecDestroy(s->graph);
   if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
   delete s;
@@ -1941,7 +1943,7 @@ struct SmallBufs {
   D4S *part, *part2;  // part2: second set for k_pair_solve
   int *late;
   unsigned long long *clk;  // loop start and budget (ns)
-  size_t bytes;
+  size_t bytes, head;  // head: bytes before the partial sums, sent to the device in one copy
   size_t size() const { return bytes; }
 };
 // partial sums per RHS: the larger of the pair kernels' blocks of ST sites and
@@ -1967,6 +1969,7 @@ static SmallBufs small_layout(void *base, int cap, int vh) {
   b.clk = cv.take<unsigned long long>(2);
   b.scale = cv.take<double>(cap);
   b.unscale = cv.take<double>(cap);
+  b.head = cv.size();
   b.part = cv.take<D4S>((size_t)cap * nbp);
   b.part2 = cv.take<D4S>(nbx <= SOLO_NBX ? (size_t)cap * nbx : 0);
   b.late = cv.take<int>(cap / 2);
@@ -1993,6 +1996,8 @@ static int sloppy_alloc(lqcd_ctx *ctx, int nrhs, int gran = 2) {
   cudaFree(s->x.e);
   cudaFree(s->r32);
   cudaFree(s->small);
+  if (s->h_small) cudaFreeHost(s->h_small);
+  s->h_small = nullptr;
   s->sd = nullptr; s->sn = nullptr; s->f32 = nullptr; s->x = FxIterate{}; s->r32 = nullptr;
   s->small = nullptr;
   s->cap = 0;
@@ -2007,6 +2012,7 @@ static int sloppy_alloc(lqcd_ctx *ctx, int nrhs, int gran = 2) {
   s->x.cap = cap;
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->r32, (size_t)cap * g.V * 6 * sizeof(float4)));
   LQCD_CUDA_TRY(ctx, cudaMalloc(&s->small, small_layout(nullptr, cap, g.Vh).size()));
+  LQCD_CUDA_TRY(ctx, cudaMallocHost(&s->h_small, small_layout(nullptr, cap, g.Vh).head));
   // padding right-hand sides of a tile are computed alongside the real ones: start them at zero
   LQCD_CUDA_TRY(ctx, cudaMemset(s->sd, 0, 7 * pairs * 6 * vh * sizeof(uint4)));
   if (!s->h_counts) LQCD_CUDA_TRY(ctx, cudaMallocHost(&s->h_counts, 16 * sizeof(int)));
@@ -2180,15 +2186,14 @@ struct MixedRun : RunIface {
   double delta = 0.05, floor2 = 4e-12;  // (2e-6)^2: inner FP32 target floor, relative to |b_inner|^2
   SF r, rhat, pp, v, s, t, tmp;
   F32F x32, b32, r32, t32, o32, res[2];  // res: outer residual by parity
-  SmallBufs sb;
+  SmallBufs sb, host;  // host: the pinned copy of sb's head
   std::vector<double> rr, bb, prev_rel, hscale, hun, have;  // have: 1 where the iterate was started
   std::vector<SState> hs;
-  std::vector<int> hl, hp, bad, hflags, keep_status;
+  std::vector<int> hl, hp, bad, hflags;
   int cycle = 0;
   const int max_cycles = 10;
   bool timed_out = false;
   int force_code = -1;  // launch code (blocks per SM * 10 + hop variant) chosen by the autotuner while it times
-  unsigned long long budget_ns = ~0ull;  // host copy of the value sent to the device (pinned lifetime: the run)
 
   MixedRun(lqcd_ctx *c, const double2 *b_, double2 *x_, int n, const lqcd_solver_params &p_, lqcd_solve_stats *s_,
            cudaStream_t st_, double t0_)
@@ -2223,6 +2228,7 @@ struct MixedRun : RunIface {
     auto f32 = [&](int k) { F32F ff; ff.d = ss->f32 + (size_t)k * cap * 6 * vh; ff.vh = vh; return ff; };
     x32 = f32(0); b32 = f32(1); r32 = f32(2); t32 = f32(3); o32 = f32(4);
     sb = small_layout(ss->small, cap, vh);
+    host = small_layout(ss->h_small, cap, vh);
     rr.assign(nrhs, 0.0);
     bb.assign(nrhs, 0.0);
     prev_rel.assign(nrhs, 1e300);
@@ -2231,7 +2237,6 @@ struct MixedRun : RunIface {
     hs.assign(cap, SState{});
     bad.assign(nrhs, 0);
     hflags.assign(cap, 0);
-    keep_status.assign(nrhs, 0);
     for (int k = 0; k < nrhs; ++k) stats[k] = lqcd_solve_stats{0, LQCD_OK, 0.0, 0, 0};
     for (int k = 0; k < 2; ++k) {
       res[k].d = ss->r32 + (size_t)k * cap * 6 * vh;
@@ -2312,6 +2317,8 @@ struct MixedRun : RunIface {
     int rc = cycle == 0 ? fp64_residual_into(ctx, b, nullptr, nullptr, nrhs, rr.data(), bb.data(), st)
                         : fx_residual(ctx, ss->x, b, res, todo.data(), (int)todo.size(), rr.data(), st);
     if (rc) return rc;
+    if (cycle > 0)  // the scalars that cycle_end asked for came with the residual
+      for (int k : todo) hs[k] = host.sc[k];
     hl.clear();
     hp.clear();
     std::fill(hflags.begin(), hflags.end(), 0);
@@ -2347,21 +2354,25 @@ struct MixedRun : RunIface {
       return LQCD_OK;
     }
     int *counts = sb.counts;
-    int hc[5] = {0, 0, (int)hl.size(), 0, (int)hp.size()};
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.cyc_list, hl.data(), hl.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.cyc_pairs, hp.data(), hp.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(counts, hc, sizeof(hc), cudaMemcpyHostToDevice, st));
     // wall-clock budget left for this cycle's inner loop, in ns (the loop's own check)
-    budget_ns = ~0ull;
+    unsigned long long budget_ns = ~0ull;
     if (p.timeout_ms > 0) {
       const double left = p.timeout_ms - (wall_ms() - t0);
       budget_ns = left > 0 ? (unsigned long long)(left * 1e6) : 0ull;
     }
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.clk + 1, &budget_ns, sizeof(budget_ns), cudaMemcpyHostToDevice, st));
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.scale, hscale.data(), cap * sizeof(double), cudaMemcpyHostToDevice, st));
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.unscale, hun.data(), cap * sizeof(double), cudaMemcpyHostToDevice, st));
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.sc, hs.data(), cap * sizeof(SState), cudaMemcpyHostToDevice, st));
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(sb.flags, hflags.data(), cap * sizeof(int), cudaMemcpyHostToDevice, st));
+    // everything the cycle needs in one copy from pinned memory (the lists in between are
+    // built on the device)
+    std::copy(hs.begin(), hs.end(), host.sc);
+    std::copy(hflags.begin(), hflags.end(), host.flags);
+    std::copy(hl.begin(), hl.end(), host.cyc_list);
+    std::copy(hp.begin(), hp.end(), host.cyc_pairs);
+    std::fill(host.counts, host.counts + 16, 0);
+    host.counts[2] = (int)hl.size();
+    host.counts[4] = (int)hp.size();
+    host.clk[1] = budget_ns;
+    std::copy(hscale.begin(), hscale.end(), host.scale);
+    std::copy(hun.begin(), hun.end(), host.unscale);
+    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(ss->small, ss->h_small, sb.head, cudaMemcpyHostToDevice, st));
     // inner right-hand side: b32 = scale (r_e + kappa H_eo r_o), o32 = scale r_o
     if (cycle == 0) {
       KL k_cvt64to32_both<<<G, ST, 0, st>>>(g, b, b32, o32, sb.scale, sb.cyc_list, counts + 2, nbx);
@@ -2515,11 +2526,7 @@ struct MixedRun : RunIface {
     if (cycle == 0)
       for (int k : hl) have[k] = 1.0;
     LQCD_LAUNCH_CHECK(ctx, "mixed: correction");
-    for (int k = 0; k < nrhs; ++k) keep_status[k] = hs[k].status;
-    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(hs.data(), sb.sc, cap * sizeof(SState), cudaMemcpyDeviceToHost, st));
-    LQCD_CUDA_TRY(ctx, cudaStreamSynchronize(st));
-    for (int k = 0; k < nrhs; ++k)
-      if (!std::binary_search(hl.begin(), hl.end(), k)) hs[k].status = keep_status[k];
+    LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(host.sc, sb.sc, cap * sizeof(SState), cudaMemcpyDeviceToHost, st));
     inner = false;
     ++cycle;
     return LQCD_OK;
