@@ -226,7 +226,8 @@ __device__ __forceinline__ void load_link32(const float4 *U, int p, int mu, int 
 }
 
 // FP32 hop in direction MU for NR right-hand sides of one site: each link is
-// loaded and reconstructed once and applied to all of them
+// loaded and reconstructed once and applied to all of them, after their neighbours
+// have been projected (half the registers of the neighbours themselves)
 template <int MU, int NR>
 __device__ __forceinline__ void hop_dir32n(const Geom &g, int p_out, const int c[4], int i, const F32F &in,
                                            const int rhs[NR], const float4 *links, float2 acc[NR][4][3]) {
@@ -235,14 +236,20 @@ __device__ __forceinline__ void hop_dir32n(const Geom &g, int p_out, const int c
     int cn[4] = {c[0], c[1], c[2], c[3]};
     cn[MU] = (c[MU] + 1 == g.L[MU]) ? 0 : c[MU] + 1;
     const int sn = site_of(g, cn);
-    load_link32(links, p_out, MU, i, g.Vh, u);
+    float2 hh[NR][2][3];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      float2 v[12], h[2][3], x[2][3], ps[4][3];
+      float2 v[12], ps[4][3];
       in.load(rhs[r], sn >> 1, v);
 #pragma unroll
       for (int k = 0; k < 12; ++k) ps[k / 3][k % 3] = v[k];
-      spin_project<MU, -1>(ps, h);
+      spin_project<MU, -1>(ps, hh[r]);
+    }
+    load_link32(links, p_out, MU, i, g.Vh, u);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      float2 x[2][3];
+      float2 (&h)[2][3] = hh[r];
       su3_mul<false>(u, h, x);
       if (MU == 3 && c[3] == g.L[3] - 1) {
 #pragma unroll
@@ -257,14 +264,20 @@ __device__ __forceinline__ void hop_dir32n(const Geom &g, int p_out, const int c
     int cn[4] = {c[0], c[1], c[2], c[3]};
     cn[MU] = (c[MU] == 0) ? g.L[MU] - 1 : c[MU] - 1;
     const int sn = site_of(g, cn);
-    load_link32(links, 1 - p_out, MU, sn >> 1, g.Vh, u);
+    float2 hh[NR][2][3];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      float2 v[12], h[2][3], x[2][3], ps[4][3];
+      float2 v[12], ps[4][3];
       in.load(rhs[r], sn >> 1, v);
 #pragma unroll
       for (int k = 0; k < 12; ++k) ps[k / 3][k % 3] = v[k];
-      spin_project<MU, +1>(ps, h);
+      spin_project<MU, +1>(ps, hh[r]);
+    }
+    load_link32(links, 1 - p_out, MU, sn >> 1, g.Vh, u);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      float2 x[2][3];
+      float2 (&h)[2][3] = hh[r];
       su3_mul<true>(u, h, x);
       if (MU == 3 && c[3] == 0) {
 #pragma unroll
@@ -398,8 +411,13 @@ __device__ __forceinline__ float2 hop32x2_site(const Geom &g, int p_out, int i, 
 // 2j + 1; with an odd count the last thread recomputes entry 2j for its second
 // slot and stores nothing for it), which halves the link loads and the
 // reconstruction of the third link row per right-hand side.  EPI_RES: partial |out|^2.
+// Bound by the latency of its loads and the FP32 pipe.  PLAIN is fastest with the
+// registers of three blocks per SM, the others, which end with more loads, with four:
+// 16^3 x 32, 384 right-hand sides, PLAIN / RES / AXPY 1.56 / 2.17 / 2.04 ms with the
+// link loaded first and four blocks, 1.39 / 2.16 / 1.81 like this (RES and AXPY with
+// three: 2.21 and 1.91).
 template <int EPI>
-__global__ void __launch_bounds__(ST, 4) k_hop32x2(Geom g, int p_out, const float4 *links, F32F in, F32F out, F32F A,
+__global__ void __launch_bounds__(ST, EPI == EPI_PLAIN ? 3 : 4) k_hop32x2(Geom g, int p_out, const float4 *links, F32F in, F32F out, F32F A,
                                                 F32F B, float cA, float cB, float cH, const int *list,
                                                 const int *count, D4S *part, int nbx) {
   const int cnt = *count;
