@@ -2664,8 +2664,8 @@ static int mixed_block(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, co
   // The graph is recorded on a stream of its own and launched on the caller's, which may
   // be the default stream.  There the first solve of a configuration launches its
   // iterations directly: recording a graph takes longer than it saves once, and a
-  // program that solves once on the default stream does not pay for it.  12 point
-  // sources of 4^4: 1.70 -> 1.20 ms, 17 sources of 8^3 x 16 (FP16): 2.94 -> 2.00 ms.
+  // program that solves once on the default stream does not pay for it.  17 sources of
+  // 8^3 x 16 (FP16): 2.94 -> 2.00 ms.
   bool solo = run->solo();
   bool use_graph = !solo && !ctx->prof_on && getenv("LQCD_NO_GRAPH") == nullptr;
   if (use_graph && (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread)) {
