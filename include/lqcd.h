@@ -127,7 +127,7 @@ const char *lqcd_last_error(const lqcd_ctx *ctx);
  * computed on).  U: [V][4][3][3] complex128, device or host pointer.  Keeps an
  * FP64 copy and the reduced-precision copies the mixed-precision solver reads:
  * FP32 reconstruct-12 (first two rows; the third is (row1 x row2)^*), FP16 with
- * all 18 reals duplicated, tf32 and double-float.  Errors: LQCD_ERR_NOT_SU3 if
+ * all 18 reals duplicated, tf32 and 58-bit integers.  Errors: LQCD_ERR_NOT_SU3 if
  * a link deviates from unitarity or unit determinant by more than 1e-12
  * (nothing is kept). */
 int lqcd_set_gauge(lqcd_ctx *ctx, const double *U, lqcd_stream_t stream);
@@ -172,8 +172,8 @@ int lqcd_solve_batch(lqcd_ctx *ctx, const double *b, double *x, int nrhs,
  * device).  lqcd_batch_run solves every entry with *params: in mixed precision
  * the inner iterations of all lattices are captured into one CUDA graph (one
  * branch per lattice) on `stream`, which must be a created stream (not the
- * legacy default); one graph launch advances every lattice by four iterations,
- * and each lattice's outer FP64 refinement runs between launches.  FP64 solves
+ * legacy default); one graph launch runs every lattice's inner solve of the
+ * current cycle, and each lattice's outer refinement runs between launches.  FP64 solves
  * the entries one after another.  stats: host array of n_stats records, one
  * per RHS in the order of lqcd_batch_add; n_stats below the batch's RHS total
  * is rejected with LQCD_ERR_INVALID before any work (lqcd_batch_rhs gives the
@@ -292,8 +292,10 @@ int lqcd_smear_ape(lqcd_ctx *ctx, double alpha, int n_iter, double *out, lqcd_st
  * within each time slice, all four spins alike (the paper uses alpha = 4,
  * n = 50).  ape_links = 1 uses the links of the last lqcd_smear_ape, 0 the
  * context's links; normalise = 1 divides each factor by (1 + 6 alpha).
- * in, out: [nrhs][V][4][3] complex128 device, distinct.  FP64.  Errors:
- * INVALID (in == out, host pointers, ape_links without lqcd_smear_ape),
+ * in, out: [nrhs][V][4][3] complex128 device, distinct.  On SU(3) links the
+ * steps run in 58-bit integer arithmetic (relative to each site and spin's
+ * colour vector; a vector with an entry that is not finite becomes NaN), else
+ * in FP64.  Errors: INVALID (in == out, host pointers, ape_links without lqcd_smear_ape),
  * NO_GAUGE. */
 int lqcd_smear_gaussian(lqcd_ctx *ctx, const double *in, double *out, int nrhs, double alpha, int n_iter,
                         int ape_links, int normalise, lqcd_stream_t stream);
