@@ -231,6 +231,12 @@ int lqcd_create(lqcd_ctx **out, const int dims[4], int device) {
     delete c;
     return cuda_error(nullptr, e, "cudaMalloc(flag)");
   }
+  e = cudaEventCreateWithFlags(&c->fx_ev, cudaEventDisableTiming);
+  if (e != cudaSuccess) {
+    cudaFree(c->d_flag);
+    delete c;
+    return cuda_error(nullptr, e, "cudaEventCreate");
+  }
   *out = c;
   return LQCD_OK;
 }

@@ -228,28 +228,23 @@ static bool capturing(cudaStream_t st) {
   if (err) cudaGetLastError();
   return err || cap != cudaStreamCaptureStatusNone;
 }
-// The workspaces of integer limbs are shared by the context's streams: a call that uses
-// one waits for the event of the last (fx_enter) and records its own (fx_leave).  Under
-// capture neither does anything: the graph's order is its program's.
-bool fx_enter(lqcd_ctx *ctx, cudaStream_t st) {
-  if (capturing(st)) return true;
-  if (!ctx->fx_ev && cudaEventCreateWithFlags(&ctx->fx_ev, cudaEventDisableTiming) != cudaSuccess) {
-    cudaGetLastError();
-    ctx->fx_ev = nullptr;
-    return false;
+FxUse::FxUse(lqcd_ctx *c, cudaStream_t s) : ok(c->gauge_su3), ctx(c), st(s) {
+  if (ctx->fx_depth++ > 0) {  // within another use, which is on the same stream
+    ok = ctx->fx_ok;
+    return;
   }
-  if (ctx->fx_used && ctx->fx_stream != st && cudaStreamWaitEvent(st, ctx->fx_ev, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  if (ok && !capturing(st)) {
+    ok = record = cudaStreamWaitEvent(st, ctx->fx_ev, 0) == cudaSuccess;
+    if (!ok) cudaGetLastError();
   }
-  return true;
+  ctx->fx_ok = ok;
 }
-int fx_leave(lqcd_ctx *ctx, cudaStream_t st) {
-  if (capturing(st)) return LQCD_OK;
-  LQCD_CUDA_TRY(ctx, cudaEventRecord(ctx->fx_ev, st));
-  ctx->fx_used = true;
-  ctx->fx_stream = st;
-  return LQCD_OK;
+FxUse::~FxUse() {
+  --ctx->fx_depth;
+  if (record && cudaEventRecord(ctx->fx_ev, st) != cudaSuccess) {  // nothing to wait for: be done first
+    cudaGetLastError();
+    cudaStreamSynchronize(st);
+  }
 }
 
 // Workspace of integer limbs for n_par parities of up to *chunk right-hand sides, or
@@ -263,7 +258,7 @@ static char *fx_workspace(lqcd_ctx *ctx, int nrhs, int n_par, int *chunk, cudaSt
   *chunk = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FX_WS_BYTES / per));
   int rc = LQCD_OK;
   void *w = workspace(ctx, WS_FX, per * *chunk, &rc);
-  return w && fx_enter(ctx, st) ? (char *)w : nullptr;
+  return (char *)w;
 }
 // one launch; fx: the input as integer limbs, or null
 static int launch_hop64_one(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
@@ -303,8 +298,9 @@ int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool o
   const Geom &g = ctx->geom;
   int chunk = 0;
   char *w = nullptr;
+  const FxUse use(ctx, st);
   // (sized for both parities: a canonical field is converted whole)
-  if (ctx->gauge_su3) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
+  if (use.ok) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
   if (!w)
     return launch_hop64_one(ctx, st, dag, in_canon, out_canon, p_out, in, in_stride, out, out_stride, A, cA, B, cB, cH,
                             active, nrhs, nullptr);
@@ -324,7 +320,7 @@ int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool o
                               A ? A + o : nullptr, cA, B ? B + o : nullptr, cB, cH, act, n, &f);
     if (rc) return rc;
   }
-  return fx_leave(ctx, st);
+  return LQCD_OK;
 }
 
 int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, bool dagger, cudaStream_t st) {
@@ -332,7 +328,8 @@ int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, b
   const size_t stride = (size_t)g.V * 12;
   int chunk = nrhs;
   char *w = nullptr;
-  if (ctx->gauge_su3) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
+  const FxUse use(ctx, st);
+  if (use.ok) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
   if (!w) chunk = nrhs;
   for (int r = 0; r < nrhs; r += chunk) {
     const int n = std::min(chunk, nrhs - r);
@@ -351,7 +348,7 @@ int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, b
       if (rc) return rc;
     }
   }
-  return w ? fx_leave(ctx, st) : LQCD_OK;
+  return LQCD_OK;
 }
 
 // --------------------------------------------------------- layout changes
@@ -1150,6 +1147,7 @@ int fp64_solve(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, const lqcd
   double t0 = wall_ms();
   size_t full = (size_t)ctx->geom.V * 12;
   int worst = LQCD_OK;
+  const FxUse use(ctx, st);  // one for all hops of the solve
   for (int k0 = 0; k0 < nrhs; k0 += blk) {
     int nk = nrhs - k0 < blk ? nrhs - k0 : blk;
     int rc = p.solver == LQCD_SOLVER_CG ? fp64_cg_block(ctx, b + k0 * full, x + k0 * full, nk, p, stats + k0, st, t0)

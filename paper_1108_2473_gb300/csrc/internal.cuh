@@ -194,9 +194,9 @@ struct lqcd_ctx {
   double2 *Uape = nullptr;    // APE-smeared copy (spatial links smeared) [V][4][3][3], on first use
   bool have_ape = false;
   std::vector<lqcd::DevBuf> ws;  // named workspaces, grow-only
-  cudaEvent_t fx_ev = nullptr;   // end of the last use of a workspace of limbs, on fx_stream
-  cudaStream_t fx_stream = nullptr;
-  bool fx_used = false;
+  cudaEvent_t fx_ev = nullptr;   // end of the last use of a workspace of limbs (FxUse)
+  int fx_depth = 0;              // uses that are open
+  bool fx_ok = false;            // the outermost one has its wait enqueued
   lqcd::SloppyState *sloppy = nullptr;
   std::string err;
   int *d_flag = nullptr;      // device error flag scratch
@@ -246,8 +246,25 @@ extern std::atomic<long long> g_launches;
 int set_error(lqcd_ctx *ctx, int code, const char *fmt, ...);
 int cuda_error(lqcd_ctx *ctx, cudaError_t e, const char *where);
 void *workspace(lqcd_ctx *ctx, int slot, size_t bytes, int *status);
-bool fx_enter(lqcd_ctx *ctx, cudaStream_t st);  // around the use of a workspace of limbs
-int fx_leave(lqcd_ctx *ctx, cudaStream_t st);
+
+// Around the use of a workspace of integer limbs on st.  The workspaces are shared by the
+// context's streams: the outermost use waits for the event of the last one and records
+// its own at its end, however it ends.  It always waits, also on the stream of the last
+// use: a handle does not tell streams apart (one that was destroyed lends it to the next,
+// and cudaStreamPerThread is another stream in each thread).  Under capture it does
+// nothing: the graph's order is its program's.
+struct FxUse {
+  FxUse(lqcd_ctx *ctx, cudaStream_t st);
+  ~FxUse();
+  FxUse(const FxUse &) = delete;
+  FxUse &operator=(const FxUse &) = delete;
+  bool ok;  // else the workspace may not be used; false also for links that are not SU(3)
+
+ private:
+  lqcd_ctx *ctx;
+  cudaStream_t st;
+  bool record = false;
+};
 bool is_device_ptr(const void *p);
 
 #define LQCD_CUDA_TRY(ctx, call)                         \

@@ -561,7 +561,8 @@ static int gauss_fx(lqcd_ctx *ctx, const double2 *U, const double2 *in, double2 
   const size_t per = 2 * (nd * sizeof(int4) + ne * sizeof(int));
   const int chunk = (int)std::max<size_t>(1, std::min<size_t>(nrhs, GAUSS_WS_BYTES / per));
   char *w = (char *)workspace(ctx, WS_SMEAR, per * chunk, &rc);
-  if (!w || !fx_enter(ctx, st)) return rc;
+  const FxUse use(ctx, st);
+  if (!w || !use.ok) return rc;
   *done = true;
   KL k_spatial_links<<<(g.V * 4 + 255) / 256, 256, 0, st>>>(g, U, links, vb);
   LQCD_LAUNCH_CHECK(ctx, "k_spatial_links");
@@ -595,7 +596,7 @@ static int gauss_fx(lqcd_ctx *ctx, const double2 *U, const double2 *in, double2 
     KL k_gauss_out<<<(unsigned)vb * n, 128, 0, st>>>(g.V, f[n_iter % 2], out + o);
     LQCD_LAUNCH_CHECK(ctx, "k_gauss_out");
   }
-  return fx_leave(ctx, st);
+  return LQCD_OK;
 }
 
 }  // namespace lqcd
@@ -621,10 +622,9 @@ extern "C" int lqcd_smear_ape(lqcd_ctx *ctx, double alpha, int n_iter, double *o
   const int threads = 128, blocks = (g.V * 4 + threads - 1) / threads;
   int4 *links = nullptr;
   const int vb = (g.V + 31) / 32;
-  if (ctx->gauge_su3 && n_iter > 0) {
+  const FxUse use(ctx, st);
+  if (use.ok && n_iter > 0)  // (without the workspace: FP64)
     links = (int4 *)workspace(ctx, WS_SMEAR_FX, (size_t)3 * vb * 288 * sizeof(int4), &rc);
-    if (links && !fx_enter(ctx, st)) links = nullptr;  // (without the workspace: FP64)
-  }
   for (int it = 0; it < n_iter; ++it) {
     double2 *dst = bufs[it % 2];
     if (links) {
@@ -636,7 +636,6 @@ extern "C" int lqcd_smear_ape(lqcd_ctx *ctx, double alpha, int n_iter, double *o
     LQCD_LAUNCH_CHECK(ctx, "k_ape_step");
     src = dst;
   }
-  if (links && (rc = fx_leave(ctx, st)) != LQCD_OK) return rc;
   if (n_iter == 0)
     LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->Uape, ctx->U64, n * sizeof(double2), cudaMemcpyDeviceToDevice, st));
   if (out) LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(out, ctx->Uape, n * sizeof(double2), cudaMemcpyDeviceToDevice, st));

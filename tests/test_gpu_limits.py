@@ -1,0 +1,61 @@
+"""Calls at the limits of what the entry points accept: several streams on one context,
+and inputs that are not finite, of extreme size or of very different size within a site."""
+import ctypes
+import threading
+
+import numpy as np
+import pytest
+
+from lattice_inputs import haar_su3_field, gaussian_spinors
+from tests._gpu import lattice, to_dev, torch
+
+pytestmark = pytest.mark.gpu
+
+
+def test_streams_share_a_context():
+    """D and Gaussian smearing of one context on several streams without a synchronisation:
+    created streams in turn, streams whose handle is that of a destroyed one with work still
+    pending, and the per-thread stream, which is another one in each thread.  The workspace
+    that they share is handed over in order: the results are those of single calls."""
+    dims, n = (8, 8, 8, 8), 64
+    with lattice(dims, haar_su3_field(dims, 41), 0.12) as (L, h):
+        x = [to_dev(gaussian_spinors(dims, 1, 42 + k).reshape(1, -1, 4, 3)).repeat(n, 1, 1, 1) for k in range(2)]
+        calls = [lambda q, o: L.lqcd_apply_dirac(h, q, o),
+                 lambda q, o: L.lqcd_smear_gaussian(h, q, o, alpha=0.5, n_iter=3, normalise=True)]
+        ref = [[torch.empty_like(q) for q in x] for _ in calls]
+        for f, r in zip(calls, ref):
+            for q, o in zip(x, r):
+                f(q, o)
+        torch.cuda.synchronize()
+
+        def compare(out):
+            torch.cuda.synchronize()
+            for c, k, o in out:
+                assert torch.equal(o, ref[c][k])
+
+        streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+        out = []
+        for k in range(8):
+            with torch.cuda.stream(streams[k % 2]):
+                out.append((k // 2 % 2, k % 2, torch.empty_like(x[0])))
+                calls[out[-1][0]](x[k % 2], out[-1][2])
+        compare(out)
+
+        rt, out = torch.cuda.cudart(), [(0, k % 2, torch.empty_like(x[0])) for k in range(8)]
+        torch.cuda.synchronize()
+        for c, k, o in out:
+            s = ctypes.c_void_p()
+            assert int(rt.cudaStreamCreate(ctypes.addressof(s))) == 0
+            with torch.cuda.stream(torch.cuda.ExternalStream(s.value)):
+                calls[c](x[k], o)
+            assert int(rt.cudaStreamDestroy(s.value)) == 0
+        compare(out)
+
+        lib, per_thread = L.load(), ctypes.c_void_p(2)  # cudaStreamPerThread
+        out = [(0, k % 2, torch.empty_like(x[0])) for k in range(8)]
+        torch.cuda.synchronize()
+        for c, k, o in out:
+            t = threading.Thread(target=lambda: lib.lqcd_apply_dirac(h, x[k].data_ptr(), o.data_ptr(), n, 0, per_thread))
+            t.start()
+            t.join()
+        compare(out)
