@@ -36,6 +36,7 @@
 // partial per (RHS, site block) and summed by one warp per RHS in a fixed
 // order: a right-hand side's arithmetic does not depend on its batch mates.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdlib>
 #include <memory>
@@ -2218,7 +2219,7 @@ struct MixedRun : RunIface {
       : ctx(c), b(b_), x(x_), nrhs(n), p(p_), stats(s_), st(st_), t0(t0_) {}
   int *dev_counts() override { return sb.counts; }
   unsigned long long *dev_clock() override { return sb.clk; }
-  int max_loops() const override { return p.max_iter + 1; }
+  int max_loops() const override { return std::min(p.max_iter, INT_MAX - 1) + 1; }
 
   int init() override {
     int rc = sloppy_alloc(ctx, nrhs, Ops::GS);
@@ -2485,7 +2486,7 @@ struct MixedRun : RunIface {
       return cudaErrorNotSupported;
     } else {
       PairSolve<SF> a{ctx->U16, ctx->U32, r, rhat, pp, v, s, t, tmp, x32, b32, r32, t32, sb.sc, sb.flags, sb.counts, sb.late,
-                      sb.act_pairs, {sb.part, sb.part2}, sb.clk, nbx, p.max_iter, p.max_iter + 1, k2, 1.f, delta * delta};
+                      sb.act_pairs, {sb.part, sb.part2}, sb.clk, nbx, p.max_iter, max_loops(), k2, 1.f, delta * delta};
       KL k_clock_start<<<1, 1, 0, q>>>(sb.counts, sb.clk);
       const int C = solo_cluster();
       auto kern = k_pair_solve<SF>;

@@ -59,3 +59,27 @@ def test_streams_share_a_context():
             t.start()
             t.join()
         compare(out)
+
+
+@pytest.mark.parametrize("dims,n", [((4, 4, 4, 4), 3), ((8, 8, 8, 16), 2)])
+def test_largest_iteration_cap(dims, n):
+    """max_iter = 2^31 - 1 ends like any other cap that is not reached: one cluster per pair
+    (4^4) and the loop of launches, on the default and on a created stream."""
+    cap = 2**31 - 1
+    with lattice(dims, haar_su3_field(dims, 43), 0.12) as (L, h):
+        b = to_dev(gaussian_spinors(dims, n, 44).reshape(n, -1, 4, 3))
+        for prec in (L.LQCD_PREC_MIXED_FP16, L.LQCD_PREC_MIXED_BF16):
+            res = []
+            for stream in (None, torch.cuda.Stream()):
+                for m in (20000, cap):
+                    x = torch.empty_like(b)
+                    with torch.cuda.stream(stream):
+                        before = L.lqcd_launch_count()
+                        rc, st = L.lqcd_solve_batch(h, b, x, L.solver_params(tol=1e-10, max_iter=m, precision=prec,
+                                                                             timeout_ms=20000.0))
+                    assert rc == 0
+                    res.append((st, x, L.lqcd_launch_count() - before))
+            for st, x, _ in res[1:]:
+                assert st == res[0][0] and torch.equal(x, res[0][1])
+            # no more kernels than with a cap that is out of reach as well
+            assert res[3][2] <= res[2][2]
