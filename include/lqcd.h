@@ -129,7 +129,9 @@ const char *lqcd_last_error(const lqcd_ctx *ctx);
  * FP32 reconstruct-12 (first two rows; the third is (row1 x row2)^*), FP16 with
  * all 18 reals duplicated, tf32 and 58-bit integers.  Errors: LQCD_ERR_NOT_SU3 if
  * a link deviates from unitarity or unit determinant by more than 1e-12
- * (nothing is kept). */
+ * (nothing is kept).  NaN entries do not count as a deviation: such a field is
+ * kept, FP64 calls then give NaN where the link enters, and solves report
+ * LQCD_ERR_NONFINITE. */
 int lqcd_set_gauge(lqcd_ctx *ctx, const double *U, lqcd_stream_t stream);
 
 /* As lqcd_set_gauge but for arbitrary complex 3x3 links (no SU(3) check).

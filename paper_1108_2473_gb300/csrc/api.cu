@@ -88,6 +88,11 @@ __global__ void k_pack_gauge(const double2 *__restrict__ U, Geom g, float4 *U32,
   for (int a = 0; a < 3; ++a)
 #pragma unroll
     for (int b = 0; b < 3; ++b) m[a][b] = u[a * 3 + b];
+  // a NaN, which the maxima below pass over, has no integer form: bit 1 of the flag
+  int top = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) top = fx_max(top, m[k / 3][k % 3]);
+  if (top >= 0x7ff00000) atomicOr(flag, 2);
   double dev = 0.0;
   for (int a = 0; a < 3; ++a)
     for (int b = 0; b < 3; ++b) {
@@ -303,14 +308,15 @@ static int set_gauge_impl(lqcd_ctx *ctx, const double *U, lqcd_stream_t stream, 
   int flag = 0;
   LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(&flag, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   LQCD_CUDA_TRY(ctx, cudaStreamSynchronize(st));
-  if (flag && require_su3) {
+  if ((flag & 1) && require_su3) {
     ctx->have_gauge = false;
     return set_error(ctx, LQCD_ERR_NOT_SU3, "lqcd_set_gauge: a link is not SU(3) within 1e-12");
   }
   LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->U64, stage, n64 * sizeof(double2), cudaMemcpyDeviceToDevice, st));
   ctx->have_gauge = true;
   ctx->have_ape = false;  // smeared links belong to the previous field
-  ctx->gauge_su3 = !flag;
+  ctx->gauge_su3 = !(flag & 1);
+  ctx->fx_links = !flag;
   int rc = pack_gauge_sloppy(ctx, st);
   if (rc != LQCD_OK) return rc;
   LQCD_CUDA_TRY(ctx, cudaStreamSynchronize(st));

@@ -228,7 +228,7 @@ static bool capturing(cudaStream_t st) {
   if (err) cudaGetLastError();
   return err || cap != cudaStreamCaptureStatusNone;
 }
-FxUse::FxUse(lqcd_ctx *c, cudaStream_t s) : ok(c->gauge_su3), ctx(c), st(s) {
+FxUse::FxUse(lqcd_ctx *c, cudaStream_t s) : ok(c->fx_links), ctx(c), st(s) {
   if (ctx->fx_depth++ > 0) {  // within another use, which is on the same stream
     ok = ctx->fx_ok;
     return;

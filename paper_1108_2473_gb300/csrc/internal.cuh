@@ -185,6 +185,7 @@ struct lqcd_ctx {
   double kappa = 0.0;
   bool have_gauge = false;
   bool gauge_su3 = false;     // links checked SU(3): reconstruct-12 copies are valid
+  bool fx_links = false;      // and finite: the integer limbs stand for them, else FP64 kernels run
   double2 *U64 = nullptr;     // canonical [V][4][3][3]
   float4 *U32 = nullptr;      // recon-12 FP32  [2 parity][4 mu][3 float4][Vh]
   uint4 *U16 = nullptr;       // FP16, all 18 reals, each twice  [2 parity][4 mu][5 uint4][Vh]
@@ -258,7 +259,7 @@ struct FxUse {
   ~FxUse();
   FxUse(const FxUse &) = delete;
   FxUse &operator=(const FxUse &) = delete;
-  bool ok;  // else the workspace may not be used; false also for links that are not SU(3)
+  bool ok;  // else the workspace may not be used; false also for links without limbs
 
  private:
   lqcd_ctx *ctx;

@@ -667,7 +667,7 @@ extern "C" int lqcd_smear_gaussian(lqcd_ctx *ctx, const double *in, double *out,
   // FP64 for links that are not SU(3), for a scale or alpha without 58-bit form, and
   // where the limbs' workspace could not be had
   int rc = LQCD_OK;
-  if (ctx->gauge_su3 && std::isnormal(scale) && (alpha == 0.0 || std::isnormal(alpha))) {
+  if (ctx->fx_links && std::isnormal(scale) && (alpha == 0.0 || std::isnormal(alpha))) {
     bool done = false;
     rc = gauss_fx(ctx, U, (const double2 *)in, (double2 *)out, nrhs, alpha, scale, n_iter, st, &done);
     if (done) return rc;

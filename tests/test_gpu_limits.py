@@ -7,7 +7,8 @@ import numpy as np
 import pytest
 
 from lattice_inputs import haar_su3_field, gaussian_spinors
-from tests._gpu import lattice, to_dev, torch
+from oracle import dirac as od
+from tests._gpu import lattice, to_dev, to_np, torch
 
 pytestmark = pytest.mark.gpu
 
@@ -83,3 +84,27 @@ def test_largest_iteration_cap(dims, n):
                 assert st == res[0][0] and torch.equal(x, res[0][1])
             # no more kernels than with a cap that is out of reach as well
             assert res[3][2] <= res[2][2]
+
+
+@pytest.mark.parametrize("mu", [0, 1, 2, 3])
+def test_nan_link_stays_nan(mu):
+    """A link with a NaN entry: D is NaN where the link enters and nowhere else, and no
+    solve reports success."""
+    dims = (4, 4, 4, 4)
+    U = haar_su3_field(dims, 5)
+    U[1, 2, 3, 0, mu, 1, 0] = np.nan
+    psi = gaussian_spinors(dims, 2, 7)
+    with np.errstate(invalid="ignore"):
+        ref = np.stack([od.apply_D(U, 0.12, psi[k]) for k in range(2)])
+    with lattice(dims, U, 0.12) as (L, h):
+        x = to_dev(psi.reshape(2, -1, 4, 3))
+        out = torch.empty_like(x)
+        L.lqcd_apply_dirac(h, x, out)
+        got = to_np(out, dims)
+        assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.isnan(ref).any()
+        fine = ~np.isnan(ref)
+        assert np.abs(got - ref)[fine].max() <= 1e-13
+        for kw in (dict(precision=L.LQCD_PREC_FP64), dict(precision=L.LQCD_PREC_FP64, solver=L.LQCD_SOLVER_CG),
+                   dict(precision=L.LQCD_PREC_MIXED_BF16), dict(precision=L.LQCD_PREC_MIXED_FP16)):
+            rc, st = L.lqcd_solve_batch(h, x, out, L.solver_params(tol=1e-10, rhs_block=2, **kw))
+            assert rc == L.LQCD_ERR_NONFINITE and all(s["status"] == rc for s in st), kw
