@@ -15,6 +15,7 @@
 
 #include "internal.cuh"
 #include "fxfield.cuh"
+#include "fpconv.cuh"
 
 namespace lqcd {
 
@@ -145,58 +146,70 @@ __device__ __forceinline__ void coords_full(const Geom &g, int s, int c[4]) {
   c[3] = r / g.L[2];
 }
 
-// one APE step: thread per (site, mu); spatial links smeared, temporal copied
-__global__ void k_ape_step(Geom g, const double2 *__restrict__ Uin, double2 *Uout, double alpha) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= g.V * 4) return;
-  const int s = idx >> 2, i = idx & 3;
-  const double2 *ui = Uin + (size_t)idx * 9;
-  if (i == 3) {
+// One APE step, thread per (site, mu): spatial links smeared, temporal copied.  only: null,
+// or nothing is done unless *only is set.
+__global__ void k_ape_step(Geom g, const double2 *__restrict__ Uin, double2 *Uout, double alpha, const int *only) {
+  if (only && !*only) return;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.V * 4; idx += gridDim.x * blockDim.x) {
+    const int s = idx >> 2, i = idx & 3;
+    const double2 *ui = Uin + (size_t)idx * 9;
+    double2 *uo = Uout + (size_t)idx * 9;
+    if (i == 3) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) Uout[(size_t)idx * 9 + k] = ui[k];
-    return;
+      for (int k = 0; k < 9; ++k) uo[k] = ui[k];
+      continue;
+    }
+    int c[4];
+    coords_full(g, s, c);
+    const M3 U = load_m3(ui);
+    M3 S;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) S.m[k / 3][k % 3] = make_double2(0.0, 0.0);
+    for (int j = 0; j < 3; ++j) {
+      if (j == i) continue;
+      const int s_j = shift_site(g, c, j, 1), s_i = shift_site(g, c, i, 1), s_mj = shift_site(g, c, j, -1);
+      int cmj[4] = {c[0], c[1], c[2], c[3]};
+      cmj[j] = (c[j] - 1 + g.L[j]) % g.L[j];
+      const int s_mj_i = shift_site(g, cmj, i, 1);
+      const M3 Uj = load_m3(Uin + ((size_t)s * 4 + j) * 9);
+      const M3 Ui_j = load_m3(Uin + ((size_t)s_j * 4 + i) * 9);
+      const M3 Uj_i = load_m3(Uin + ((size_t)s_i * 4 + j) * 9);
+      const M3 up = mm<false, true>(mm<false, false>(Uj, Ui_j), Uj_i);  // U_j(x) U_i(x+j) U_j(x+i)^+
+      const M3 Uj_mj = load_m3(Uin + ((size_t)s_mj * 4 + j) * 9);
+      const M3 Ui_mj = load_m3(Uin + ((size_t)s_mj * 4 + i) * 9);
+      const M3 Uj_mji = load_m3(Uin + ((size_t)s_mj_i * 4 + j) * 9);
+      const M3 dn = mm<false, false>(mm<true, false>(Uj_mj, Ui_mj), Uj_mji);  // U_j(x-j)^+ U_i(x-j) U_j(x-j+i)
+#pragma unroll
+      for (int k = 0; k < 9; ++k) S.m[k / 3][k % 3] = cadd(S.m[k / 3][k % 3], cadd(up.m[k / 3][k % 3], dn.m[k / 3][k % 3]));
+    }
+    M3 V;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) V.m[k / 3][k % 3] = make_double2(fma(alpha, S.m[k / 3][k % 3].x, U.m[k / 3][k % 3].x), fma(alpha, S.m[k / 3][k % 3].y, U.m[k / 3][k % 3].y));
+    store_m3(uo, project_su3(V));
   }
-  int c[4];
-  coords_full(g, s, c);
-  const M3 U = load_m3(ui);
-  M3 S;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) S.m[k / 3][k % 3] = make_double2(0.0, 0.0);
-  for (int j = 0; j < 3; ++j) {
-    if (j == i) continue;
-    const int s_j = shift_site(g, c, j, 1), s_i = shift_site(g, c, i, 1), s_mj = shift_site(g, c, j, -1);
-    int cmj[4] = {c[0], c[1], c[2], c[3]};
-    cmj[j] = (c[j] - 1 + g.L[j]) % g.L[j];
-    const int s_mj_i = shift_site(g, cmj, i, 1);
-    const M3 Uj = load_m3(Uin + ((size_t)s * 4 + j) * 9);
-    const M3 Ui_j = load_m3(Uin + ((size_t)s_j * 4 + i) * 9);
-    const M3 Uj_i = load_m3(Uin + ((size_t)s_i * 4 + j) * 9);
-    const M3 up = mm<false, true>(mm<false, false>(Uj, Ui_j), Uj_i);  // U_j(x) U_i(x+j) U_j(x+i)^+
-    const M3 Uj_mj = load_m3(Uin + ((size_t)s_mj * 4 + j) * 9);
-    const M3 Ui_mj = load_m3(Uin + ((size_t)s_mj * 4 + i) * 9);
-    const M3 Uj_mji = load_m3(Uin + ((size_t)s_mj_i * 4 + j) * 9);
-    const M3 dn = mm<false, false>(mm<true, false>(Uj_mj, Ui_mj), Uj_mji);  // U_j(x-j)^+ U_i(x-j) U_j(x-j+i)
-#pragma unroll
-    for (int k = 0; k < 9; ++k) S.m[k / 3][k % 3] = cadd(S.m[k / 3][k % 3], cadd(up.m[k / 3][k % 3], dn.m[k / 3][k % 3]));
-  }
-  M3 V;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) V.m[k / 3][k % 3] = make_double2(fma(alpha, S.m[k / 3][k % 3].x, U.m[k / 3][k % 3].x), fma(alpha, S.m[k / 3][k % 3].y, U.m[k / 3][k % 3].y));
-  store_m3(Uout + (size_t)idx * 9, project_su3(V));
 }
 
 // integer limbs of the spatial links, [3 directions][block of 32 sites][9][32] int4;
-// thread per (site, mu)
-__global__ void k_spatial_links(Geom g, const double2 *__restrict__ U, int4 *out, int vb) {
+// thread per (site, mu).  *bad is set where a link has none: its rows and columns are not
+// of length 1, as after the projection of a singular matrix, which is NaN.  FP64 arithmetic
+// is then taken everywhere.
+__global__ void k_spatial_links(Geom g, const double2 *__restrict__ U, int4 *out, int vb, int *bad) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const int s = idx >> 2, mu = idx & 3;
   if (s >= g.V || mu == 3) return;
   int4 *o = out + ((size_t)mu * vb + (s >> 5)) * 288 + (s & 31);
+  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const double2 u = U[(size_t)idx * 9 + k];
     o[32 * k] = fx_link_entry(u.x, u.y);
+    const float re = f64_to_f32_bits(u.x), im = f64_to_f32_bits(u.y), n = fmaf(re, re, im * im);
+    row[k / 3] += n;
+    col[k % 3] += n;
   }
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    if (!(fabsf(row[k] - 1.f) < 0x1p-8f && fabsf(col[k] - 1.f) < 0x1p-8f)) *bad = 1;  // (also NaN)
 }
 
 // One APE step for SU(3) links: the staples, columns of three-link products, on the
@@ -290,32 +303,25 @@ __global__ void __launch_bounds__(128) k_ape_step_fx(Geom g, const double2 *__re
   for (int k = 0; k < 9; ++k) uo[k] = V.m[k / 3][k % 3];
 }
 
-// One Gaussian step in FP64 of the spin row `spin` of one site: q + alpha (H q).
-__device__ __noinline__ void gauss_site64(const Geom &g, const double2 *__restrict__ U, const double2 *__restrict__ in,
-                                          int s, int spin, double alpha, double2 out[3]) {
+// Component a of one Gaussian step in FP64 at site s: q + alpha (H q)
+__device__ __forceinline__ double2 gauss_row64(const Geom &g, const double2 *__restrict__ U,
+                                               const double2 *__restrict__ q, int s, int a, double alpha) {
   int c[4];
   coords_full(g, s, c);
-  double2 acc[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) acc[k] = make_double2(0.0, 0.0);
+  double2 acc = make_double2(0.0, 0.0);
+  int stride = 1;
+#pragma unroll 1
   for (int i = 0; i < 3; ++i) {
-    const int sf = shift_site(g, c, i, 1), sb = shift_site(g, c, i, -1);
-    const double2 *uf = U + ((size_t)s * 4 + i) * 9;   // U_i(x)
-    const double2 *ub = U + ((size_t)sb * 4 + i) * 9;  // U_i(x - i)
-    const double2 *qf = in + (size_t)sf * 12 + spin * 3, *qb = in + (size_t)sb * 12 + spin * 3;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        acc[a] = cmac(acc[a], uf[a * 3 + b], qf[b]);   // U_i(x)[a][b] q(x+i)
-        acc[a] = cmacc(acc[a], ub[b * 3 + a], qb[b]);  // conj(U_i(x-i)[b][a]) q(x-i)
-      }
+    const int L = g.L[i], ci = i == 0 ? c[0] : (i == 1 ? c[1] : c[2]);
+    const int sf = s + (ci + 1 == L ? stride * (1 - L) : stride), sb = s + (ci == 0 ? stride * (L - 1) : -stride);
+    stride *= L;
+#pragma unroll 1
+    for (int b = 0; b < 3; ++b) {
+      acc = cmac(acc, U[((size_t)s * 4 + i) * 9 + a * 3 + b], q[(size_t)sf * 12 + b]);    // U_i(x)[a][b] q(x+i)
+      acc = cmacc(acc, U[((size_t)sb * 4 + i) * 9 + b * 3 + a], q[(size_t)sb * 12 + b]);  // conj(U_i(x-i)[b][a]) q(x-i)
+    }
   }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const double2 q = in[(size_t)s * 12 + spin * 3 + k];
-    out[k] = make_double2(fma(alpha, acc[k].x, q.x), fma(alpha, acc[k].y, q.y));
-  }
+  return make_double2(fma(alpha, acc.x, q[(size_t)s * 12 + a].x), fma(alpha, acc.y, q[(size_t)s * 12 + a].y));
 }
 
 // The n Gaussian steps on integer limbs (fx64.cuh), for SU(3) links: the source is
@@ -330,7 +336,7 @@ __device__ __noinline__ void gauss_site64(const Geom &g, const double2 *__restri
 // GAUSS_NAN one that is not finite.
 // Links: [3 directions][block of 32 sites][9][32] int4.
 constexpr int GAUSS_SH = 5;  // six directions of |X| < 2.45 * 2^58 stay below 2^62 (gauss_mul)
-constexpr int GAUSS_ZERO = -(1 << 28), GAUSS_NAN = 1 << 28;
+constexpr int GAUSS_ZERO = -(1 << 28), GAUSS_NAN = 1 << 28, GAUSS_FP64 = 1 << 29;
 struct GaussF {
   int4 *d;
   int *e;
@@ -341,12 +347,24 @@ struct GaussF {
   __device__ int *exp(int rhs, int spin, int s) const { return e + (size_t)(rhs * 4 + spin) * vb * 32 + s; }
 };
 
+// Where links have no limbs (*bad, k_spatial_links) every exponent is GAUSS_FP64, and the
+// three kernels below work on FP64 fields in the same memory, [rhs][V][12] double2.
+__device__ __forceinline__ double2 *gauss_fp64(const GaussF &f, int V, int rhs) {
+  return (double2 *)f.d + (size_t)rhs * V * 12;
+}
+
 // FP64 -> limbs; a block takes 32 sites, a warp one spin
-__global__ void __launch_bounds__(128) k_gauss_in(int V, const double2 *__restrict__ in, GaussF f) {
+__global__ void __launch_bounds__(128) k_gauss_in(int V, const double2 *__restrict__ in, GaussF f, const int *bad) {
   const int rhs = blockIdx.x / f.vb, s = (blockIdx.x % f.vb) * 32 + (threadIdx.x & 31), spin = threadIdx.x >> 5;
   if (s >= V) return;
   const double2 *q = in + ((size_t)rhs * V + s) * 12 + spin * 3;
   const double2 v[3] = {q[0], q[1], q[2]};
+  if (*bad) {
+    *f.exp(rhs, spin, s) = GAUSS_FP64;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gauss_fp64(f, V, rhs)[(size_t)s * 12 + spin * 3 + k] = v[k];
+    return;
+  }
   const int m = fx_max(fx_max(fx_max(0, v[0]), v[1]), v[2]);
   unsigned low = 0u;
 #pragma unroll
@@ -377,6 +395,11 @@ __global__ void __launch_bounds__(128) k_gauss_out(int V, GaussF f, double2 *__r
   const int E = *f.exp(rhs, spin, s);
   const int4 *q = f.at(rhs, spin, s);
   double2 *o = out + ((size_t)rhs * V + s) * 12 + spin * 3;
+  if (E == GAUSS_FP64) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) o[k] = gauss_fp64(f, V, rhs)[(size_t)s * 12 + spin * 3 + k];
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     if (E == GAUSS_ZERO) {
@@ -437,7 +460,8 @@ __device__ __forceinline__ void gauss_dir(const int4 *__restrict__ link, const i
 // neighbours are mostly zero, 9.8 ms with each neighbour converted where it is used and
 // 3.6 ms here (6.4 while the links of zero neighbours were loaded).
 __global__ void __launch_bounds__(128, 4) k_gauss_step(Geom g, const int4 *__restrict__ U, GaussF in, GaussF out,
-                                                       GaussCoef alpha, GaussCoef scale, bool scaled) {
+                                                       GaussCoef alpha, GaussCoef scale, bool scaled,
+                                                       const double2 *__restrict__ U64, double alpha64, double scale64) {
   const int vb = in.vb, lane = threadIdx.x & 31, spin = threadIdx.x >> 5;
   const int blk = blockIdx.x % vb, rhs = blockIdx.x / vb;
   const int site = blk * 32 + lane, s = min(site, g.V - 1);
@@ -455,6 +479,15 @@ __global__ void __launch_bounds__(128, 4) k_gauss_step(Geom g, const int4 *__res
   int Em = GAUSS_ZERO;
 #pragma unroll
   for (int q = 0; q < 6; ++q) Em = max(Em, *in.exp(rhs, spin, n[q]));
+  if (E0 == GAUSS_FP64) {  // rolled: this rare branch shall not take registers from the other
+    if (site >= g.V) return;
+    *out.exp(rhs, spin, s) = GAUSS_FP64;
+    const double2 *q = gauss_fp64(in, g.V, rhs) + spin * 3;
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k)
+      gauss_fp64(out, g.V, rhs)[(size_t)s * 12 + spin * 3 + k] = cscale(gauss_row64(g, U64, q, s, k, alpha64), scale64);
+    return;
+  }
   if (E0 == GAUSS_ZERO && Em == GAUSS_ZERO) {  // (the values of a zero vector are not read)
     if (site < g.V) *out.exp(rhs, spin, s) = GAUSS_ZERO;
     return;
@@ -527,10 +560,10 @@ __global__ void k_gauss_step64(Geom g, const double2 *__restrict__ U, const doub
   if (idx >= (size_t)nrhs * g.V * 4) return;
   const int s = (int)((idx >> 2) % g.V), spin = (int)(idx & 3);
   const size_t rhs = (idx >> 2) / g.V;
-  double2 v[3];
-  gauss_site64(g, U, in + rhs * g.V * 12, s, spin, alpha, v);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) out[(rhs * g.V + s) * 12 + spin * 3 + k] = cscale(v[k], scale);
+#pragma unroll 1
+  for (int k = 0; k < 3; ++k)
+    out[(rhs * g.V + s) * 12 + spin * 3 + k] =
+        cscale(gauss_row64(g, U, in + rhs * g.V * 12 + spin * 3, s, k, alpha), scale);
 }
 
 // c + lo as 58 bits below c's exponent, |lo| at most half a unit in the last place of c
@@ -548,13 +581,27 @@ static GaussCoef gauss_coef(double c, double lo = 0.0) {
 // L2 run before the next ones start, so that the steps read and write L2.
 constexpr size_t GAUSS_WS_BYTES = 64u << 20;
 
+// workspace for the limbs of the spatial links and the flag of k_spatial_links
+static int4 *spatial_limbs(lqcd_ctx *ctx, int vb, int **bad, int *rc) {
+  Carver sizing(nullptr);
+  sizing.take<int4>((size_t)3 * vb * 288);
+  sizing.take<int>(1);
+  void *w = workspace(ctx, WS_SMEAR_FX, sizing.size(), rc);
+  if (!w) return nullptr;
+  Carver cv(w);
+  int4 *links = cv.take<int4>((size_t)3 * vb * 288);
+  *bad = cv.take<int>(1);
+  return links;
+}
+
 // *done: false if the workspace was refused, and nothing was launched
 static int gauss_fx(lqcd_ctx *ctx, const double2 *U, const double2 *in, double2 *out, int nrhs, double alpha,
                     double scale, int n_iter, cudaStream_t st, bool *done) {
   const Geom &g = ctx->geom;
   const int vb = (g.V + 31) / 32;
   int rc = LQCD_OK;
-  int4 *links = (int4 *)workspace(ctx, WS_SMEAR_FX, (size_t)3 * vb * 288 * sizeof(int4), &rc);
+  int *bad = nullptr;
+  int4 *links = spatial_limbs(ctx, vb, &bad, &rc);
   *done = false;
   if (!links) return rc;
   const size_t nd = (size_t)4 * vb * 96, ne = (size_t)4 * vb * 32;  // per right-hand side
@@ -564,7 +611,8 @@ static int gauss_fx(lqcd_ctx *ctx, const double2 *U, const double2 *in, double2 
   const FxUse use(ctx, st);
   if (!w || !use.ok) return rc;
   *done = true;
-  KL k_spatial_links<<<(g.V * 4 + 255) / 256, 256, 0, st>>>(g, U, links, vb);
+  LQCD_CUDA_TRY(ctx, cudaMemsetAsync(bad, 0, sizeof(int), st));
+  KL k_spatial_links<<<(g.V * 4 + 255) / 256, 256, 0, st>>>(g, U, links, vb, bad);
   LQCD_LAUNCH_CHECK(ctx, "k_spatial_links");
   GaussF f[2];
   for (int k = 0; k < 2; ++k) {
@@ -587,10 +635,11 @@ static int gauss_fx(lqcd_ctx *ctx, const double2 *U, const double2 *in, double2 
   for (int r = 0; r < nrhs; r += chunk) {
     const int n = std::min(chunk, nrhs - r);
     const size_t o = (size_t)r * g.V * 12;
-    KL k_gauss_in<<<(unsigned)vb * n, 128, 0, st>>>(g.V, in + o, f[0]);
+    KL k_gauss_in<<<(unsigned)vb * n, 128, 0, st>>>(g.V, in + o, f[0], bad);
     LQCD_LAUNCH_CHECK(ctx, "k_gauss_in");
     for (int it = 0; it < n_iter; ++it) {
-      KL k_gauss_step<<<(unsigned)vb * n, 128, 0, st>>>(g, links, f[it % 2], f[1 - it % 2], ca, cs, scaled);
+      KL k_gauss_step<<<(unsigned)vb * n, 128, 0, st>>>(g, links, f[it % 2], f[1 - it % 2], ca, cs, scaled, U,
+                                                          alpha, scale);
       LQCD_LAUNCH_CHECK(ctx, "k_gauss_step");
     }
     KL k_gauss_out<<<(unsigned)vb * n, 128, 0, st>>>(g.V, f[n_iter % 2], out + o);
@@ -621,17 +670,22 @@ extern "C" int lqcd_smear_ape(lqcd_ctx *ctx, double alpha, int n_iter, double *o
   const double2 *src = ctx->U64;
   const int threads = 128, blocks = (g.V * 4 + threads - 1) / threads;
   int4 *links = nullptr;
+  int *bad = nullptr;
   const int vb = (g.V + 31) / 32;
   const FxUse use(ctx, st);
   if (use.ok && n_iter > 0)  // (without the workspace: FP64)
-    links = (int4 *)workspace(ctx, WS_SMEAR_FX, (size_t)3 * vb * 288 * sizeof(int4), &rc);
+    links = spatial_limbs(ctx, vb, &bad, &rc);
+  if (links) LQCD_CUDA_TRY(ctx, cudaMemsetAsync(bad, 0, sizeof(int), st));
   for (int it = 0; it < n_iter; ++it) {
     double2 *dst = bufs[it % 2];
     if (links) {
-      KL k_spatial_links<<<(g.V * 4 + 255) / 256, 256, 0, st>>>(g, src, links, vb);
+      KL k_spatial_links<<<(g.V * 4 + 255) / 256, 256, 0, st>>>(g, src, links, vb, bad);
       KL k_ape_step_fx<<<dim3((g.V + 127) / 128, 4), 128, 0, st>>>(g, src, links, vb, dst, alpha);
+      // in place of what links without limbs gave (in the kernel above, the branch and its
+      // registers made a step on 16^3 x 32 10% slower)
+      KL k_ape_step<<<std::min(blocks, 512), threads, 0, st>>>(g, src, dst, alpha, bad);
     } else {
-      KL k_ape_step<<<blocks, threads, 0, st>>>(g, src, dst, alpha);
+      KL k_ape_step<<<blocks, threads, 0, st>>>(g, src, dst, alpha, nullptr);
     }
     LQCD_LAUNCH_CHECK(ctx, "k_ape_step");
     src = dst;

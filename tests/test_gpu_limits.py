@@ -108,3 +108,53 @@ def test_nan_link_stays_nan(mu):
                    dict(precision=L.LQCD_PREC_MIXED_BF16), dict(precision=L.LQCD_PREC_MIXED_FP16)):
             rc, st = L.lqcd_solve_batch(h, x, out, L.solver_params(tol=1e-10, rhs_block=2, **kw))
             assert rc == L.LQCD_ERR_NONFINITE and all(s["status"] == rc for s in st), kw
+
+
+def _singular_field(dims):
+    """A field whose x link at one site is one, as are the links of its four spatial staples:
+    U + alpha S = 0 there for alpha = -1/4, and its projection is NaN."""
+    U = haar_su3_field(dims, 6)
+    t, z, y, x = 1, 2, 1, 0
+    one = np.eye(3)
+    lx, ly, lz, _ = dims
+    U[t, z, y, x, 0] = one
+    for dz, dy in ((0, 1), (0, -1), (1, 0), (-1, 0)):
+        zz, yy = (z + dz) % lz, (y + dy) % ly
+        U[t, zz, yy, x, 0] = one
+        mu = 1 if dy else 2
+        for xx in (x, (x + 1) % lx):
+            if dy + dz > 0:
+                U[t, z, y, xx, mu] = one
+            else:
+                U[t, zz, yy, xx, mu] = one
+    return U
+
+
+@pytest.mark.parametrize("dims", [(4, 4, 4, 4), (6, 4, 4, 2)])
+@pytest.mark.parametrize("steps", [1, 2, 3])
+def test_nan_smeared_links_stay_nan(dims, steps):
+    """APE links that are NaN: later APE steps and Gaussian smearing give NaN where, and only
+    where, FP64 arithmetic gives it (a temporal link that is not SU(3) selects it; smearing
+    does not read it)."""
+    U = _singular_field(dims)
+    q = gaussian_spinors(dims, 2, 8).reshape(2, -1, 4, 3)
+    q[1] = 0.0
+    q[1, 5, 2, 1] = 1.0  # most vectors zero
+    res = []
+    for general in (True, False):
+        with lattice(dims, kappa=0.12) as (L, h):
+            W = U.copy()
+            if general:
+                W[0, 0, 0, 0, 3] *= 2.0
+            u = to_dev(W.reshape(-1))
+            L.lqcd_set_gauge_general(h, u)
+            links, src = torch.empty_like(u), to_dev(q)
+            out = torch.empty_like(src)
+            L.lqcd_smear_ape(h, -0.25, steps, links)
+            L.lqcd_smear_gaussian(h, src, out, alpha=0.7, n_iter=2, ape_links=True, normalise=True)
+            links = links.reshape(-1, 4, 9)[:, :3].contiguous()
+            res.append((links.cpu().numpy(), out.cpu().numpy()))
+    for a, b in zip(*res):
+        assert np.isnan(a).any() and np.array_equal(np.isnan(a), np.isnan(b))
+        fine = ~np.isnan(a)
+        assert np.abs(a - b)[fine].max() <= 1e-9
