@@ -86,8 +86,9 @@ __device__ __forceinline__ M3 inv_dag(const M3 &a, double2 det) {
 
 // projection onto SU(3): unitary polar factor by the Newton iteration
 // X <- (z X + X^{-+} / z) / 2, then the det phase removed.  z = |det X|^{-1/3} speeds
-// up the first steps and does not change the limit: it is formed in FP32, and is 1 once
-// |det X| is within 2^-10 of 1.
+// up the first steps and does not change the limit: it is formed in FP32, from the
+// determinant divided by a power of two where its square leaves the range of FP32, and is
+// 1 once |det X| is within 2^-10 of 1.
 // Bound by the FP64 pipe, so the iteration is written for few FP64 operations: one
 // reciprocal per step, the size of a step read off the high words of its differences
 // by integer maxima, and no iteration after one that moved X by less than 2^-27: the
@@ -99,10 +100,19 @@ __device__ M3 project_su3(M3 x) {
     const double2 d = det3(x);
     const float ad = sqrtf((float)d.x * (float)d.x + (float)d.y * (float)d.y);
     double hz = 0.5, hzi = 0.5;
-    if (fabsf(ad - 1.f) > 0x1p-10f && ad > 0.f && ad < 1e30f) {
-      const float z = cbrtf(1.f / ad);
-      hz = 0.5 * z;
-      hzi = 0.5f / z;
+    if (!(fabsf(ad - 1.f) <= 0x1p-10f)) {
+      const int e = (max(__double2hiint(d.x) & 0x7fffffff, __double2hiint(d.y) & 0x7fffffff) >> 20) - 1023;
+      if (ad > 0x1p-60f && ad < 0x1p60f) {
+        const float z = cbrtf(1.f / ad);
+        hz = 0.5 * z;
+        hzi = 0.5f / z;
+      } else if (e > -1023 && e < 1024) {  // det = (x0 + i y0) 2^(3 q), of size 1 to 12
+        const int q = (e + 1023) / 3 - 341;
+        const double f = __hiloint2double((1023 - q) << 20, 0);
+        const float x0 = (float)(d.x * f * f * f), y0 = (float)(d.y * f * f * f), z = cbrtf(rsqrtf(x0 * x0 + y0 * y0));
+        hz = z * __hiloint2double((1022 - q) << 20, 0);
+        hzi = __hiloint2double((1022 + q) << 20, 0) / z;
+      }
     }
     const M3 y = inv_dag(x, d);
     int diff = 0;  // high word of the largest |component| of the step

@@ -6,8 +6,9 @@ import threading
 import numpy as np
 import pytest
 
-from lattice_inputs import haar_su3_field, gaussian_spinors
+from lattice_inputs import eps_su3_field, haar_su3_field, gaussian_spinors
 from oracle import dirac as od
+from oracle import smear as osm
 from tests._gpu import lattice, to_dev, to_np, torch
 
 pytestmark = pytest.mark.gpu
@@ -158,3 +159,17 @@ def test_nan_smeared_links_stay_nan(dims, steps):
         assert np.isnan(a).any() and np.array_equal(np.isnan(a), np.isnan(b))
         fine = ~np.isnan(a)
         assert np.abs(a - b)[fine].max() <= 1e-9
+
+
+@pytest.mark.parametrize("alpha", [1e6, 1e9, -1e9, 1e14, 1e40])
+def test_ape_large_alpha(alpha):
+    """The projection onto SU(3) of sums far above 1, whose determinants leave the range
+    of FP32: the tolerance of the same field at alpha = 0.5."""
+    dims = (4, 6, 4, 4)
+    U = eps_su3_field(dims, 0.5, 3)
+    V = int(np.prod(dims))
+    with lattice(dims, U, 0.12) as (L, h):
+        out = torch.empty(V * 36, dtype=torch.complex128, device="cuda")
+        L.lqcd_smear_ape(h, alpha, 2, out)
+        got = out.cpu().numpy().reshape(U.shape)
+    assert np.max(np.abs(got - osm.ape_smear(U, alpha, 2))) < 1e-12
