@@ -12,6 +12,7 @@
 // right-hand sides of 16^3 x 32, now 10.2; the update of the iterate 4.5 ms, now 2.7
 // and 4.9 ms for the first and the later ones, without clearing it before.)
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "fxfield.cuh"
@@ -100,13 +101,15 @@ __global__ void __launch_bounds__(ST) k_fx_accum(F32F e0, F32F e1, FxF x0, FxF x
 // per block.  A block takes 64 sites of one listed right-hand side (lane layout of
 // fxf_hop); blocks are ordered (chunk of FXR_CHUNK right-hand sides, site block,
 // right-hand side in the chunk), so that blocks issued together share their links.
-// kappa = (kh 2^29 + kl) 2^(ek - 1080).
+// kappa = (kh 2^29 + kl) 2^(ek - 1080).  r is stored, and summed, times 2^shift[slot]
+// (about one over the last residual): FP32 would hold neither the residual of sources of
+// any size nor its square.
 constexpr int FXR_SITES = 64;
 constexpr int FXR_CHUNK = 8;
 __global__ void __launch_bounds__(2 * FXR_SITES, 4) k_fx_resid(Geom g, int p_out, const int4 *__restrict__ U, FxF xin,
                                                             FxF xown, const double2 *__restrict__ b, F32F r, int kh,
-                                                            int kl, int ek, const int *list, int n, double *part,
-                                                            int nblk) {
+                                                            int kl, int ek, const int *list, const int *shift, int n,
+                                                            double *part, int nblk) {
   const int in_chunk = blockIdx.x % FXR_CHUNK, rest = blockIdx.x / FXR_CHUNK;
   const int blk = rest % nblk, slot = (rest / nblk) * FXR_CHUNK + in_chunk;
   if (slot >= n) return;  // ragged last chunk: the whole block leaves together
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(2 * FXR_SITES, 4) k_fx_resid(Geom g, int p_out
   const int Er = max(max(Ey, Ex), max(Eb, FX_EMIN));
   const int dx = min(Er - Ex, 63), dy = min(Er - Ey, 63);
   // r = I 2^(Er - 1079); FP32 as two power-of-two factors
-  const float2 f = pow2_pair(Er - 1079);
+  const float2 f = pow2_pair(Er - 1079 + shift[slot]);
   const int4 *xs = xo.site(i);
   float2 v[6];
   float rn = 0.f;
@@ -251,8 +254,8 @@ int fx_join(lqcd_ctx *ctx, const FxIterate &x, const double *have, double2 *out,
   return LQCD_OK;
 }
 
-int fx_residual(lqcd_ctx *ctx, const FxIterate &x, const double2 *b, const F32F r[2], const int *list, int n, double *rr,
-                cudaStream_t st) {
+int fx_residual(lqcd_ctx *ctx, const FxIterate &x, const double2 *b, const F32F r[2], const int *list,
+                const int *shift, int n, double *rr, cudaStream_t st) {
   if (n <= 0) return LQCD_OK;
   const Geom &g = ctx->geom;
   const int nblk = (g.Vh + FXR_SITES - 1) / FXR_SITES;
@@ -260,14 +263,16 @@ int fx_residual(lqcd_ctx *ctx, const FxIterate &x, const double2 *b, const F32F 
   Carver sizing(nullptr);
   sizing.take<double>((size_t)n * 2 * nblk);
   sizing.take<double>((size_t)n);
-  sizing.take<int>((size_t)n);
+  sizing.take<int>(2 * (size_t)n);
   void *w = workspace(ctx, WS_F64_PART, sizing.size(), &rc);
   if (!w) return rc;
   Carver cv(w);
   double *part = cv.take<double>((size_t)n * 2 * nblk);
   double *d_rr = cv.take<double>((size_t)n);
-  int *d_list = cv.take<int>((size_t)n);
-  LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(d_list, list, n * sizeof(int), cudaMemcpyHostToDevice, st));
+  int *d_list = cv.take<int>(2 * (size_t)n);
+  std::vector<int> up(list, list + n);
+  up.insert(up.end(), shift, shift + n);
+  LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(d_list, up.data(), 2 * n * sizeof(int), cudaMemcpyHostToDevice, st));
   // kappa as 58 bits below its exponent
   unsigned long long kb;
   const double kappa = ctx->kappa;
@@ -280,8 +285,8 @@ int fx_residual(lqcd_ctx *ctx, const FxIterate &x, const double2 *b, const F32F 
   const long long blocks = (long long)((n + FXR_CHUNK - 1) / FXR_CHUNK) * nblk * FXR_CHUNK;
   for (int p = 0; p < 2; ++p) {
     KL k_fx_resid<<<(unsigned)blocks, 2 * FXR_SITES, 0, st>>>(g, p, ctx->Ufx, fx_parity(x, 1 - p, g.Vh),
-                                                              fx_parity(x, p, g.Vh), b, r[p], kh, kl, ek, d_list, n,
-                                                              part, nblk);
+                                                              fx_parity(x, p, g.Vh), b, r[p], kh, kl, ek, d_list, d_list + n,
+                                                              n, part, nblk);
     LQCD_LAUNCH_CHECK(ctx, "k_fx_resid");
   }
   KL k_fx_resid_fin<<<n, 32, 0, st>>>(part, 2 * nblk, d_rr);
@@ -289,7 +294,7 @@ int fx_residual(lqcd_ctx *ctx, const FxIterate &x, const double2 *b, const F32F 
   std::vector<double> h(n);
   LQCD_CUDA_TRY(ctx, cudaMemcpyAsync(h.data(), d_rr, n * sizeof(double), cudaMemcpyDeviceToHost, st));
   LQCD_CUDA_TRY(ctx, cudaStreamSynchronize(st));
-  for (int j = 0; j < n; ++j) rr[list[j]] = h[j];
+  for (int j = 0; j < n; ++j) rr[list[j]] = std::ldexp(h[j], -2 * shift[j]);
   return LQCD_OK;
 }
 

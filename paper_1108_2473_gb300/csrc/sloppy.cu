@@ -2326,15 +2326,17 @@ struct MixedRun : RunIface {
     // at x = 0 the residual is b itself (FP64 norms only); later: b - D x on the
     // integer units for the right-hand sides corrected in the previous cycle (the
     // others' iterates, and so their residuals, have not changed)
-    std::vector<int> todo;
+    std::vector<int> todo, shift;  // shift: power of two that brings the last residual's norm near 1
     if (cycle == 0) {
       todo.resize(nrhs);
       for (int k = 0; k < nrhs; ++k) todo[k] = k;
     } else {
       todo = hl;
+      for (int k : todo) shift.push_back(-std::ilogb(rr[k]) / 2);
     }
     int rc = cycle == 0 ? fp64_residual_into(ctx, b, nullptr, nullptr, nrhs, rr.data(), bb.data(), st)
-                        : fx_residual(ctx, ss->x, b, res, todo.data(), (int)todo.size(), rr.data(), st);
+                        : fx_residual(ctx, ss->x, b, res, todo.data(), shift.data(), (int)todo.size(), rr.data(),
+                                      st);
     if (rc) return rc;
     if (cycle > 0)  // the scalars that cycle_end asked for came with the residual
       for (int k : todo) hs[k] = host.sc[k];
@@ -2343,7 +2345,8 @@ struct MixedRun : RunIface {
     std::fill(hflags.begin(), hflags.end(), 0);
     std::fill(hscale.begin(), hscale.end(), 0.0);
     std::fill(hun.begin(), hun.end(), 0.0);
-    for (int k : todo) {
+    for (size_t j = 0; j < todo.size(); ++j) {
+      const int k = todo[j];
       double rel = bb[k] > 0 ? std::sqrt(rr[k] / bb[k]) : 0.0;
       stats[k].true_rel_residual = rel;
       stats[k].iterations = hs[k].iters;
@@ -2362,7 +2365,7 @@ struct MixedRun : RunIface {
       if (status == LQCD_OK && rel > p.tol) {
         hl.push_back(k);
         if (hp.empty() || hp.back() != k / Ops::GS) hp.push_back(k / Ops::GS);
-        hscale[k] = 1.0 / std::sqrt(rr[k]);
+        hscale[k] = std::ldexp(1.0 / std::sqrt(rr[k]), cycle > 0 ? -shift[j] : 0);
         hun[k] = std::sqrt(rr[k]);
         hs[k].target2 = 0.25 * p.tol * p.tol * bb[k] / rr[k];
         hflags[k] = FLAG_RU;  // marks the members whose inner source is loaded below

@@ -52,10 +52,10 @@ struct FxIterate {
 // x = scale e (first) or x += scale e (even and odd parts) for the listed right-hand sides
 int fx_accum(lqcd_ctx *ctx, const FxIterate &x, const F32F &e, const F32F &o, const double *scale, bool first,
              const int *list, const int *count, int G, cudaStream_t st);
-// r[parity] = b - D x in FP32 for the right-hand sides list[0..n) (host list); rr
-// (host, indexed by right-hand side) receives |r|^2.  Synchronises st.
-int fx_residual(lqcd_ctx *ctx, const FxIterate &x, const double2 *b, const F32F r[2], const int *list, int n, double *rr,
-                cudaStream_t st);
+// r[parity] = 2^shift (b - D x) in FP32 for the right-hand sides list[0..n) (host list, with
+// their shifts); rr (host, indexed by right-hand side) receives |b - D x|^2.  Synchronises st.
+int fx_residual(lqcd_ctx *ctx, const FxIterate &x, const double2 *b, const F32F r[2], const int *list,
+                const int *shift, int n, double *rr, cudaStream_t st);
 // canonical FP64 x (device array have: 0 for right-hand sides whose x is zero)
 int fx_join(lqcd_ctx *ctx, const FxIterate &x, const double *have, double2 *out, int nrhs, cudaStream_t st);
 

@@ -173,3 +173,24 @@ def test_ape_large_alpha(alpha):
         L.lqcd_smear_ape(h, alpha, 2, out)
         got = out.cpu().numpy().reshape(U.shape)
     assert np.max(np.abs(got - osm.ape_smear(U, alpha, 2))) < 1e-12
+
+
+@pytest.mark.parametrize("prec", ["fp16", "bf16"])
+@pytest.mark.parametrize("scale", [1e-100, 1e-30, 1e-18, 1e26, 1e100])
+def test_mixed_solve_scaled_sources(prec, scale):
+    """Sources of any overall size beside one of size 1: the FP64 residual meets the tolerance,
+    and the reported one (FP32 components) is that residual."""
+    dims, tol = (4, 4, 4, 8), 1e-10
+    b = gaussian_spinors(dims, 3, 9).reshape(3, -1, 4, 3) * np.array([1.0, scale, -scale])[:, None, None, None]
+    with lattice(dims, haar_su3_field(dims, 10), 0.13) as (L, h):
+        p = L.LQCD_PREC_MIXED_FP16 if prec == "fp16" else L.LQCD_PREC_MIXED_BF16
+        bd = to_dev(b)
+        x, y = torch.empty_like(bd), torch.empty_like(bd)
+        rc, st = L.lqcd_solve_batch(h, bd, x, L.solver_params(tol=tol, precision=p))
+        L.lqcd_apply_dirac(h, x, y)
+        s = torch.tensor([1.0, scale, scale], dtype=torch.float64, device="cuda").reshape(3, 1, 1, 1)
+        rel = [float(torch.linalg.vector_norm(((y - bd) / s)[k]) / torch.linalg.vector_norm((bd / s)[k])) for k in range(3)]
+        assert rc == 0
+        for k in range(3):
+            assert 0.0 < rel[k] <= 1.01 * tol
+            assert abs(st[k]["true_rel_residual"] - rel[k]) <= 0.01 * rel[k]
