@@ -151,7 +151,11 @@ int lqcd_plaquette(lqcd_ctx *ctx, double *plaq, lqcd_stream_t stream);
 
 /* out = D in (dagger = 0) or D^+ in (dagger != 0) in FP64 on the full lattice,
  * for nrhs fields [nrhs][V][4][3] complex128 (device).  in and out must not
- * overlap. */
+ * overlap.  On SU(3) links the products run in 58-bit integer arithmetic: each
+ * spin row of out is rounded relative to the largest component of the input's
+ * rows that enter it, as in FP64 arithmetic (colours of a row are not told
+ * apart).  While the stream is being captured FP64 arithmetic is used, which
+ * rounds differently in the last bits. */
 int lqcd_apply_dirac(lqcd_ctx *ctx, const double *in, double *out, int nrhs, int dagger,
                      lqcd_stream_t stream);
 

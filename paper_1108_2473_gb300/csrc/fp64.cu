@@ -125,6 +125,67 @@ __device__ __noinline__ void hop_site64(const Geom &g, int p_out, int i, int hs,
   }
 }
 
+// The same by a whole warp (all lanes call, with one site; every lane receives the rows):
+// lane 4 q + a forms colour a of neighbour q = 2 mu + (0 forward, 1 backward), 48 FP64
+// operations in sequence and so about 3,000 cycles, where one lane alone takes 55,000.
+constexpr int HOP_WARP_SITES = 16;  // as many of a warp's sites take less time like this
+template <bool DAG, bool IN_CANON>
+__device__ __noinline__ void hop_site64_warp(const Geom &g, int p_out, int i, int hs, const double2 *in, const double2 *U,
+                                             double2 out[6]) {
+  const int lane = threadIdx.x & 31, q = lane >> 2, a = min(lane & 3, 2), mu = q >> 1;
+  const bool fwd = !(q & 1);
+  int c[4];
+  coords_of(g, p_out, i, c);
+  const int s = site_of(g, c);
+  int sn = s, stride = 1;
+  bool edge = false;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int L = g.L[m];
+    if (m == mu) {
+      edge = fwd ? c[m] + 1 == L : c[m] == 0;
+      sn = s + (fwd ? (edge ? stride * (1 - L) : stride) : (edge ? stride * (L - 1) : -stride));
+    }
+    stride *= L;
+  }
+  const double2 *p = in + (size_t)(IN_CANON ? sn : (sn >> 1)) * 12;
+  const double2 *u = U + ((size_t)(fwd ? s : sn) * 4 + mu) * 9;
+  const bool minus = fwd != DAG, imag = !(mu & 1);  // projector 1 -+ gamma_mu; its phases
+  const bool wrap = mu == 3 && edge;
+  // U h_r for row r = 0, 1 of the projection: h_r = psi_r + phase psi_low
+  auto eps = [&](int r) { return minus != ((mu == 1 && r == 0) || (mu == 2 && r == 1)); };  // phase < 0
+  auto half = [&](int r) {
+    const int low = mu < 2 ? 3 - r : 2 + r;
+    const bool neg = eps(r);
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const double2 x = p[r * 3 + b], y = p[low * 3 + b], t = imag ? cmuli(y) : y;
+      double2 w = u[fwd ? a * 3 + b : b * 3 + a];
+      if (!fwd) w.y = -w.y;
+      acc = cmac(acc, w, neg ? csub(x, t) : cadd(x, t));
+    }
+    if (wrap) acc = make_double2(-acc.x, -acc.y);
+    return acc;
+  };
+  const int rl = mu < 2 ? 1 - hs : hs;  // row 2 + hs is the conjugate phase of h_rl
+  double2 up = half(hs), lo = half(rl);
+  if (imag) lo = make_double2(lo.y, -lo.x);
+  if (eps(rl)) lo = make_double2(-lo.x, -lo.y);
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    up.x += __shfl_xor_sync(0xffffffffu, up.x, o);
+    up.y += __shfl_xor_sync(0xffffffffu, up.y, o);
+    lo.x += __shfl_xor_sync(0xffffffffu, lo.x, o);
+    lo.y += __shfl_xor_sync(0xffffffffu, lo.y, o);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    out[k] = make_double2(__shfl_sync(0xffffffffu, up.x, k), __shfl_sync(0xffffffffu, up.y, k));
+    out[3 + k] = make_double2(__shfl_sync(0xffffffffu, lo.x, k), __shfl_sync(0xffffffffu, lo.y, k));
+  }
+}
+
 // out = cA A + cB B + cH v at rows hs and 2 + hs (v) of one site, o: its row hs
 __device__ __forceinline__ void hop64_store(const double2 v[6], size_t o, double2 *out, const double2 *A, double cA,
                                             const double2 *B, double cB, double cH) {
@@ -165,17 +226,17 @@ __global__ void __launch_bounds__(128) k_fx_from64(Geom g, const double2 *__rest
   const double2 *q = in + (size_t)rhs * in_stride + (size_t)idx * 12;
   const FxF f = (p ? f1 : f0).at(rhs);
   double2 v[12];
-  int m = 0;
-  unsigned low = 0u;
+  int m[4] = {0, 0, 0, 0};
+  unsigned low[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
   for (int k = 0; k < 12; ++k) v[k] = q[k];
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
-    m = fx_max(m, v[k]);
-    low |= __double2loint(v[k].x) | __double2loint(v[k].y);
+    m[k / 3] = fx_max(m[k / 3], v[k]);
+    low[k / 3] |= __double2loint(v[k].x) | __double2loint(v[k].y);
   }
-  const int E = fx_site_exp(m, low);
-  f.e[i] = E;
+  const int E = fx_site_exp(max(max(m[0], m[1]), max(m[2], m[3])), low[0] | low[1] | low[2] | low[3]);
+  f.e[i] = E > 0 ? fx_with_rows(E, m, low) : E;
   if (E <= 0) return;  // the limbs of such a site are not read
   int4 *o = f.site(i);
 #pragma unroll
@@ -185,10 +246,12 @@ __global__ void __launch_bounds__(128) k_fx_from64(Geom g, const double2 *__rest
 
 // The hopping term with its SU(3) products on the integer units (fx64.cuh), on a field
 // of integer limbs (fxfield.cuh); the FP64 field `in` it was made from serves the sites
-// that have no integer form.  D on 12 right-hand sides of 16^3 x 32, conversion
-// included: 2.63 ms in FP64 arithmetic (k_hop64), 1.31 ms when each neighbour is
-// converted where it is used, 0.97 ms here; one right-hand side of 4^4: 28 us, as
-// in FP64.
+// that have no integer form or whose rows are of very different size.  D on 12
+// right-hand sides of 16^3 x 32, conversion included: 2.63 ms in FP64 arithmetic
+// (k_hop64), 1.31 ms when each neighbour is converted where it is used, 1.00 ms here;
+// one right-hand side of 4^4: 32 us.  Near a point source some sites always have such
+// rows: with each of them left to its lane 768 point sources of 4^4 took 5.44 ms to
+// solve, by whole warps 5.07 (4.74 without a look at the rows).
 template <bool DAG, bool IN_CANON, bool OUT_CANON>
 __global__ void __launch_bounds__(128, 4) k_hop64_fxf(Geom g, int p_out, const double2 *__restrict__ U,
                                                       const int4 *__restrict__ Ufx, FxF f,
@@ -201,18 +264,30 @@ __global__ void __launch_bounds__(128, 4) k_hop64_fxf(Geom g, int p_out, const d
   long long up[6], low[6];
   int Em;
   bool bad;
-  fxf_hop<DAG>(g, p_out, i, hs, f.at(rhs), Ufx, up, low, Em, bad);
-  if (site >= g.Vh) return;
+  fxf_hop<DAG, true>(g, p_out, i, hs, f.at(rhs), Ufx, up, low, Em, bad);
   double2 v[6];
-  if (bad) {
-    hop_site64<DAG, IN_CANON>(g, p_out, i, hs, in + (size_t)rhs * in_stride, U, v);
-  } else {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      v[k] = make_double2(fx_double<FXF_SH>(up[2 * k], Em), fx_double<FXF_SH>(up[2 * k + 1], Em));
-      v[3 + k] = make_double2(fx_double<FXF_SH>(low[2 * k], Em), fx_double<FXF_SH>(low[2 * k + 1], Em));
+  for (int k = 0; k < 3; ++k) {
+    v[k] = make_double2(fx_double<FXF_SH>(up[2 * k], Em), fx_double<FXF_SH>(up[2 * k + 1], Em));
+    v[3 + k] = make_double2(fx_double<FXF_SH>(low[2 * k], Em), fx_double<FXF_SH>(low[2 * k + 1], Em));
+  }
+  bad = bad && site < g.Vh;
+  unsigned todo = __ballot_sync(0xffffffffu, bad);
+  if (__popc(todo) > HOP_WARP_SITES) {
+    if (bad) hop_site64<DAG, IN_CANON>(g, p_out, i, hs, in + (size_t)rhs * in_stride, U, v);
+    todo = 0u;
+  }
+  while (todo) {
+    const int src = __ffs(todo) - 1;
+    todo &= todo - 1;
+    double2 w[6];
+    hop_site64_warp<DAG, IN_CANON>(g, p_out, __shfl_sync(0xffffffffu, i, src), hs, in + (size_t)rhs * in_stride, U, w);
+    if ((threadIdx.x & 31) == src) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) v[k] = w[k];
     }
   }
+  if (site >= g.Vh) return;
   size_t s = i;
   if (OUT_CANON) {
     int c[4];

@@ -6,7 +6,10 @@
 //   field of one parity: [rhs][block][12][32] int4, complex k = 3 spin + colour of a
 //     site as (re.h, re.l, im.h, im.l), and [rhs][block][32] int, its biased exponent
 //     E: a component is (h 2^29 + l) 2^(E - 1075 - FXF_SH), below 2^(53 + FXF_SH) in
-//     size.  E = 0 marks a site of zeros, FX_BAD one that is not finite or out of range;
+//     size.  E = 0 marks a site of zeros, FX_BAD one that is not finite or out of range.
+//     A field that FP64 arithmetic is to be matched on (k_fx_from64) has above the
+//     exponent's 11 bits how far each spin row's largest component lies below it, 5 bits
+//     a row (FX_ROW_ZERO: a row of zeros);
 //   links: [2 parity][4 mu][block][9][32] int4, the sign of the time boundary folded in.
 //
 // A site is converted once, not by each of its eight neighbours; the hopping term
@@ -22,6 +25,12 @@ namespace lqcd {
 
 constexpr int FXF_SH = 4;  // eight directions of |X| < 2.45 * 2 * 2^57 stay below 2^63
 constexpr int FX_BAD = -1;
+constexpr int FX_ROW_ZERO = 31;
+// Output rows whose largest contribution lies more than 2^FX_ROW_BITS below the stencil's
+// largest component, to which all limbs are aligned, are evaluated in FP64: rows 0 and 1 do
+// not mix, so FP64 arithmetic rounds relative to each.  The limbs' rounding is about
+// 2^-55.5 of the stencil's largest component, that of FP64 arithmetic 2^-52.5 of the row's.
+constexpr int FX_ROW_BITS = 3;
 
 __host__ __device__ inline int fx_blocks(int vh) { return (vh + 31) / 32; }
 
@@ -44,6 +53,18 @@ __device__ __forceinline__ int fx_site_exp(int m, unsigned low) {
   const int E = m >> 20;
   if (m == 0 && low == 0u) return 0;
   return (E < FX_EMIN || E > FX_EMAX) ? FX_BAD : E;
+}
+// E > 0 with its rows, m[a]: high word of the largest component of row a, low[a]: OR of its low words
+__device__ __forceinline__ int fx_with_rows(int E, const int m[4], const unsigned low[4]) {
+  int w = E;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+    w |= (m[a] == 0 && low[a] == 0u ? FX_ROW_ZERO : min(E - (m[a] >> 20), FX_ROW_ZERO - 1)) << (11 + 5 * a);
+  return w;
+}
+__device__ __forceinline__ int fx_row_exp(int w, int E, int a) {  // 0 for a row of zeros
+  const int d = (w >> (11 + 5 * a)) & 31;
+  return d == FX_ROW_ZERO ? 0 : E - d;
 }
 __device__ __forceinline__ int4 fx_split_c(long long re, long long im) {
   int4 q;
@@ -142,11 +163,13 @@ __device__ __forceinline__ void fxf_half(int p_out, int i, int vh, const int n[8
 // sites, warps 2, 3 of the next 32 (so hs is a compile-time constant of each warp's
 // code, which an SM sub-partition sees only one half of; the directions are a loop of
 // two to keep that code small).  Every thread takes part.
-// bad: a neighbour has no integer form.
+// bad: a neighbour has no integer form, or (ROWS) one of the two rows lies too far below
+// Em for the limbs (FX_ROW_BITS); the rows that enter them are those of the projections,
+// 0 with 3 and 1 with 2 for mu = x, y, 0 with 2 and 1 with 3 for z, t.
 // Per direction 108 multiply-adds on one integer pipe and about 130 adds and shifts on
 // the other, half of whose rate it reaches; 16, 20 or 24 resident warps per SM, rolled
 // or unrolled directions all took within 4% of the same time.
-template <bool DAG>
+template <bool DAG, bool ROWS>
 __device__ __forceinline__ void fxf_hop(const Geom &g, int p_out, int i, int hs, const FxF &in,
                                         const int4 *__restrict__ U, long long up[6], long long low[6], int &Em,
                                         bool &bad) {
@@ -165,11 +188,25 @@ __device__ __forceinline__ void fxf_hop(const Geom &g, int p_out, int i, int hs,
     n[2 * mu + 1] = (s + (c[mu] == 0 ? stride * (L - 1) : -stride)) >> 1;
     stride *= L;
   }
+  int xy[2] = {0, 0}, zt[2] = {0, 0};  // largest exponents of the projections' two rows
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    En[q] = in.e[n[q]];
+    const int w = in.e[n[q]];
+    En[q] = ROWS && w > 0 ? w & 0x7ff : w;
     Em = max(Em, En[q]);
-    bad = bad || En[q] < 0;
+    bad = bad || w < 0;
+    if (ROWS) {
+      int *m = q < 4 ? xy : zt;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const int h = q < 4 ? (a == 1 || a == 2) : a & 1;
+        m[h] = max(m[h], fx_row_exp(w, En[q], a));
+      }
+    }
+  }
+  if (ROWS) {
+    const int r0 = max(hs ? xy[1] : xy[0], hs ? zt[1] : zt[0]), r1 = max(hs ? xy[0] : xy[1], hs ? zt[1] : zt[0]);
+    bad = bad || (r0 > 0 && r0 < Em - FX_ROW_BITS) || (r1 > 0 && r1 < Em - FX_ROW_BITS);
   }
 #pragma unroll
   for (int k = 0; k < 6; ++k) up[k] = low[k] = 0;

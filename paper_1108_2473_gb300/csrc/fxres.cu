@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(2 * FXR_SITES, 4) k_fx_resid(Geom g, int p_out
   long long up[6], low[6];
   int Em;
   bool bad;
-  fxf_hop<false>(g, p_out, i, hs, xin.at(rhs), U, up, low, Em, bad);
+  fxf_hop<false, false>(g, p_out, i, hs, xin.at(rhs), U, up, low, Em, bad);
   int c[4];
   coords_of(g, p_out, i, c);
   const double2 *bp = b + ((size_t)rhs * g.V + site_of(g, c)) * 12;
