@@ -1,7 +1,7 @@
 // The iterate of the mixed solver and its true residual b - D x.
 //
 // The iterate is held as integer limbs with one exponent per site (fxfield.cuh: 57
-// bits relative to the site's largest component), so that the residual that
+// bits relative to the site's largest component, which every update restores), so that the residual that
 // certifies |M x - b| / |b| (Sec. III) runs on the integer units, exactly but for
 // the last of those bits, and reads the iterate in coalesced parity order.  The FP64
 // source b is brought to the same form where it is read; the residual goes out in
@@ -9,13 +9,14 @@
 // error of one evaluation is a few 1e-16 of |x|, far below the 1e-10 residual it
 // certifies.  (In double-float arithmetic, pairs of FP32 numbers, it took about
 // 10,500 FP32 operations per site and kept 48 bits: 12.1 ms per parity for 384
-// right-hand sides of 16^3 x 32, now 10.2; the update of the iterate 4.5 ms, now 2.7
-// and 4.9 ms for the first and the later ones, without clearing it before.)
+// right-hand sides of 16^3 x 32, now 10.2; the update of the iterate 4.5 ms, now 2.6
+// and 3.7 ms for the first and the later ones, without clearing it before.)
 #include <algorithm>
 #include <cmath>
 #include <vector>
 
 #include "fxfield.cuh"
+#include "fxaccum.cuh"
 #include "fpconv.cuh"
 #include "sloppy.cuh"
 
@@ -28,70 +29,48 @@ __device__ __forceinline__ float2 pow2_pair(int k) {
 }
 
 // ------------------------------------------------------------------ update
-// One complex pair of reals of x += scale e: v (FP32) as 30 bits below the site's
-// largest exponent ee, times the 58-bit scale.
-__device__ __forceinline__ long long accum_term(float v, int ee, int sh, int sl) {
-  const unsigned u = __float_as_uint(v);
-  const int ex = (u >> 23) & 0xff;
-  int m = ex ? (int)(((u & 0x7fffffu) | 0x800000u) << 6) >> min(ee - ex, 31) : 0;
-  m = (int)u < 0 ? -m : m;
-  return (fx_mad(m, sh, 0) + ((fx_mad(m, sl, 0) + (1ll << 28)) >> 29)) >> 2;
-}
-
-// x = scale e (first) or x += scale e for the listed right-hand sides, both parities.
-// Bound by memory: 288 B (first) or 480 B per site and right-hand side.
-__global__ void __launch_bounds__(ST) k_fx_accum(F32F e0, F32F e1, FxF x0, FxF x1, const double *scale, bool first,
+// x = scale e (FIRST) or x += scale e for the listed right-hand sides, both parities
+// (fxaccum.cuh).  Bound by memory, 288 B (FIRST) or 480 B per site and right-hand side,
+// and by the registers of a site's 24 sums, which are normalised together: 96 right-hand
+// sides of 16^3 x 32 take 0.66 and 0.91 ms (5 and 4 blocks per SM; 0.75 and 1.00 ms with
+// the registers that the compiler wants, 0.55 and 0.87 without normalisation).
+template <bool FIRST>
+__global__ void __launch_bounds__(ST, FIRST ? 5 : 4) k_fx_accum(F32F e0, F32F e1, FxF x0, FxF x1, const double *scale,
                                                  const int *list, const int *count, int nbx, int vh) {
   const int n_items = *count * nbx;
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     const int rhs = list[w / nbx];
     const int i = (w % nbx) * ST + threadIdx.x;
     if (i >= vh) continue;
-    const unsigned long long sb = (unsigned long long)__double_as_longlong(scale[rhs]);  // > 0
-    const int es = (int)(sb >> 52);
-    int sh, sl;
-    fx_split((long long)((sb & 0xfffffffffffffull) | 0x10000000000000ull) << 5, sh, sl);
-#pragma unroll
+    const FxScale s = fx_scale(scale[rhs]);  // > 0
+#pragma unroll 1
     for (int p = 0; p < 2; ++p) {
       const FxF x = (p ? x1 : x0).at(rhs);
       int4 *xs = x.site(i);
       const float4 *q = (p ? e1 : e0).d + (size_t)rhs * 6 * vh + i;
-      float4 v[6];
-      int m = 0;
+      float e[24];
+      long long v[24];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) v[k] = q[(size_t)k * vh];
-#pragma unroll
-      for (int k = 0; k < 6; ++k)
-        m = max(max(m, max(__float_as_int(v[k].x) & 0x7fffffff, __float_as_int(v[k].y) & 0x7fffffff)),
-                max(__float_as_int(v[k].z) & 0x7fffffff, __float_as_int(v[k].w) & 0x7fffffff));
-      const int ee = m >> 23;
-      // |scale e| < 2^(E - 1022)
-      int E = ee + es - 126;
-      if (ee == 0 || E < FX_EMIN) E = 0;
-      if (ee == 0xff || es >= 0x7ff || E > FX_EMAX) E = FX_BAD;
-      const int old = first ? 0 : x.e[i];
-      int En = E > 0 && old > 0 ? max(E, old) + 1 : max(E, old);
-      if (E < 0 || old < 0 || En > FX_EMAX) En = FX_BAD;
-      const int d_new = min(En - E, 63), d_old = min(En - old, 63);
-      if (En > 0 || first) {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-          const float2 f = (k & 1) ? make_float2(v[k >> 1].z, v[k >> 1].w) : make_float2(v[k >> 1].x, v[k >> 1].y);
-          long long re = 0, im = 0;
-          if (En > 0 && E > 0) {
-            re = accum_term(f.x, ee, sh, sl) >> d_new;
-            im = accum_term(f.y, ee, sh, sl) >> d_new;
-          }
-          int4 *o = xs + 32 * k;
-          if (!first && old > 0) {
-            const int4 t = *o;
-            re += fx_value(t.x, t.y) >> d_old;
-            im += fx_value(t.z, t.w) >> d_old;
-          }
-          *o = fx_split_c(re, im);
-        }
+      for (int k = 0; k < 6; ++k) {
+        const float4 t = q[(size_t)k * vh];
+        e[4 * k] = t.x;
+        e[4 * k + 1] = t.y;
+        e[4 * k + 2] = t.z;
+        e[4 * k + 3] = t.w;
       }
-      x.e[i] = En;
+      const int old = FIRST ? 0 : x.e[i];
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        int4 t = make_int4(0, 0, 0, 0);
+        if (!FIRST && old > 0) t = xs[32 * k];
+        v[2 * k] = fx_value(t.x, t.y);
+        v[2 * k + 1] = fx_value(t.z, t.w);
+      }
+      const int E = fx_accum_site(e, s, old, v);
+      x.e[i] = E;
+      if (E <= 0) continue;  // the limbs of such a site are not read
+#pragma unroll
+      for (int k = 0; k < 12; ++k) xs[32 * k] = fx_split_c(v[2 * k], v[2 * k + 1]);
     }
   }
 }
@@ -239,8 +218,10 @@ static FxF fx_parity(const FxIterate &x, int p, int vh) {
 int fx_accum(lqcd_ctx *ctx, const FxIterate &x, const F32F &e, const F32F &o, const double *scale, bool first,
              const int *list, const int *count, int G, cudaStream_t st) {
   const int vh = ctx->geom.Vh;
-  KL k_fx_accum<<<G, ST, 0, st>>>(e, o, fx_parity(x, 0, vh), fx_parity(x, 1, vh), scale, first, list, count,
-                                  (vh + ST - 1) / ST, vh);
+  const FxF x0 = fx_parity(x, 0, vh), x1 = fx_parity(x, 1, vh);
+  const int nbx = (vh + ST - 1) / ST;
+  if (first) KL k_fx_accum<true><<<G, ST, 0, st>>>(e, o, x0, x1, scale, list, count, nbx, vh);
+  else KL k_fx_accum<false><<<G, ST, 0, st>>>(e, o, x0, x1, scale, list, count, nbx, vh);
   LQCD_LAUNCH_CHECK(ctx, "k_fx_accum");
   return LQCD_OK;
 }
