@@ -317,6 +317,7 @@ static int set_gauge_impl(lqcd_ctx *ctx, const double *U, lqcd_stream_t stream, 
   ctx->have_ape = false;  // smeared links belong to the previous field
   ctx->gauge_su3 = !(flag & 1);
   ctx->fx_links = !flag;
+  if (ctx->fx_links) fx_reserve(ctx);
   int rc = pack_gauge_sloppy(ctx, st);
   if (rc != LQCD_OK) return rc;
   LQCD_CUDA_TRY(ctx, cudaStreamSynchronize(st));

@@ -322,18 +322,28 @@ FxUse::~FxUse() {
   }
 }
 
-// Workspace of integer limbs for n_par parities of up to *chunk right-hand sides, or
-// null (then the caller takes FP64 arithmetic, as for links that are not SU(3), which
-// may be of any size): as many as keep it in L2 (FX_WS_BYTES), at least one.  Not while
-// the stream is being captured, when nothing may be allocated.
+// Workspace of integer limbs for both parities of some right-hand sides: as many as keep it
+// in L2 (FX_WS_BYTES), at least one and at most FX_WS_RHS.  It is reserved with the gauge
+// field: D enqueues its work and allocates nothing.
 constexpr size_t FX_WS_BYTES = 96u << 20;
-static char *fx_workspace(lqcd_ctx *ctx, int nrhs, int n_par, int *chunk, cudaStream_t st) {
-  if (capturing(st)) return nullptr;
-  const size_t per = (size_t)n_par * fx_blocks(ctx->geom.Vh) * 32 * (12 * sizeof(int4) + sizeof(int));
-  *chunk = (int)std::max<size_t>(1, std::min<size_t>(nrhs, FX_WS_BYTES / per));
+constexpr size_t FX_WS_RHS = 1024;
+static size_t fx_rhs_bytes(const lqcd_ctx *ctx) {
+  return (size_t)2 * fx_blocks(ctx->geom.Vh) * 32 * (12 * sizeof(int4) + sizeof(int));
+}
+static int fx_max_chunk(const lqcd_ctx *ctx) {
+  return (int)std::max<size_t>(1, std::min(FX_WS_RHS, FX_WS_BYTES / fx_rhs_bytes(ctx)));
+}
+void fx_reserve(lqcd_ctx *ctx) {
   int rc = LQCD_OK;
-  void *w = workspace(ctx, WS_FX, per * *chunk, &rc);
-  return (char *)w;
+  workspace(ctx, WS_FX, fx_rhs_bytes(ctx) * fx_max_chunk(ctx), &rc);  // (if refused: FP64 arithmetic)
+}
+// The workspace and how many right-hand sides it takes at a time, or null: where it was
+// refused, and while the stream is being captured, when the caller takes FP64 arithmetic
+// (a graph's replays are not ordered with other uses).
+static char *fx_workspace(lqcd_ctx *ctx, int nrhs, int *chunk, cudaStream_t st) {
+  if (capturing(st)) return nullptr;
+  *chunk = std::min(nrhs, fx_max_chunk(ctx));
+  return (char *)ctx->ws[WS_FX].p;
 }
 // one launch; fx: the input as integer limbs, or null
 static int launch_hop64_one(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool out_canon, int p_out,
@@ -374,8 +384,7 @@ int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool o
   int chunk = 0;
   char *w = nullptr;
   const FxUse use(ctx, st);
-  // (sized for both parities: a canonical field is converted whole)
-  if (use.ok) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
+  if (use.ok) w = fx_workspace(ctx, nrhs, &chunk, st);
   if (!w)
     return launch_hop64_one(ctx, st, dag, in_canon, out_canon, p_out, in, in_stride, out, out_stride, A, cA, B, cB, cH,
                             active, nrhs, nullptr);
@@ -404,7 +413,7 @@ int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, b
   int chunk = nrhs;
   char *w = nullptr;
   const FxUse use(ctx, st);
-  if (use.ok) w = fx_workspace(ctx, nrhs, 2, &chunk, st);
+  if (use.ok) w = fx_workspace(ctx, nrhs, &chunk, st);
   if (!w) chunk = nrhs;
   for (int r = 0; r < nrhs; r += chunk) {
     const int n = std::min(chunk, nrhs - r);

@@ -247,6 +247,7 @@ extern std::atomic<long long> g_launches;
 int set_error(lqcd_ctx *ctx, int code, const char *fmt, ...);
 int cuda_error(lqcd_ctx *ctx, cudaError_t e, const char *where);
 void *workspace(lqcd_ctx *ctx, int slot, size_t bytes, int *status);
+void fx_reserve(lqcd_ctx *ctx);  // workspace of limbs of the FP64 hopping term
 
 // Around the use of a workspace of integer limbs on st.  The workspaces are shared by the
 // context's streams: the outermost use waits for the event of the last one and records

@@ -233,3 +233,16 @@ def test_dirac_rows_of_different_size(rows, share, dims):
             # up to 50 FP64 roundings of 2^-53 of that, here and in the oracle: below 1e-14
             err = np.abs(to_np(out, dims) - ref).max(-1)
             assert np.all(err <= 1e-14 * _row_max(psi))
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (8, 8, 8, 8)])
+def test_first_dirac_allocates_nothing(dims):
+    """The first D on a context enqueues work only: what it needs came with the gauge field."""
+    with lattice(dims, haar_su3_field(dims, 13), 0.12) as (L, h):
+        x = to_dev(gaussian_spinors(dims, 2, 14).reshape(2, -1, 4, 3))
+        out = torch.empty_like(x)
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        L.lqcd_apply_dirac(h, x, out)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
