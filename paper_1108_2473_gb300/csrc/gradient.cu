@@ -56,6 +56,12 @@ __global__ void k_adj_source(Geom g, const double2 *__restrict__ src, const doub
            ((unsigned)__double2hiint(v[k].y) << 1) | (unsigned)__double2loint(v[k].y);
     o[k] = make_double2(0.0, 0.0);
   }
+  // (a coefficient that is not finite makes its whole time slice NaN)
+#pragma unroll
+  for (int gi = 0; gi < 6; ++gi) {
+    const double2 c = coef[t * 6 + gi];
+    any |= (unsigned)(((__double2hiint(c.x) & 0x7fffffff) >= 0x7ff00000) | ((__double2hiint(c.y) & 0x7fffffff) >= 0x7ff00000));
+  }
   if (any != 0u)
 #pragma unroll
   for (int gi = 0; gi < 6; ++gi) {

@@ -246,3 +246,21 @@ def test_first_dirac_allocates_nothing(dims):
         L.lqcd_apply_dirac(h, x, out)
         torch.cuda.synchronize()
         assert torch.cuda.mem_get_info()[0] == free
+
+
+def test_gradient_nan_coefficient():
+    """A NaN coefficient of a time slice without sources is not lost: 0 NaN = NaN."""
+    dims = (4, 4, 4, 4)
+    src = np.zeros((2, 256, 4, 3), dtype=np.complex128)
+    src[0, 3, 1, 2] = src[1, 9, 0, 0] = 1.0  # time slice 0
+    with lattice(dims, haar_su3_field(dims, 15), 0.12) as (L, h):
+        s = to_dev(src)
+        sol = torch.empty_like(s)
+        prm = L.solver_params(tol=1e-10, precision=L.LQCD_PREC_FP64, rhs_block=2)
+        assert L.lqcd_solve_batch(h, s, sol, prm)[0] == 0
+        coef = np.ones((4, 6), dtype=np.complex128)
+        dU = torch.zeros(256 * 36, dtype=torch.complex128, device="cuda")
+        assert L.lqcd_gradient(h, s, sol, coef, prm, dU=dU)[1] == 0
+        coef[2, 3] = np.nan  # a slice without sources
+        _, rc, st = L.lqcd_gradient(h, s, sol, coef, prm, dU=dU)
+        assert rc == L.LQCD_ERR_NONFINITE and all(q["status"] == rc for q in st)
