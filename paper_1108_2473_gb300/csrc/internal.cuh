@@ -285,7 +285,7 @@ bool is_device_ptr(const void *p);
 enum WsSlot {
   WS_STAGE_IN = 0, WS_STAGE_OUT, WS_STAGE_AUX,
   WS_F64_VECS, WS_F64_SCAL, WS_F64_PART, WS_F64_FULL,
-  WS_LOOP_PART, WS_GRAD, WS_GRAD2, WS_SMEAR, WS_SMEAR_LINKS, WS_SMEAR_FX, WS_FX,
+  WS_LOOP_PART, WS_GRAD, WS_GRAD2, WS_SMEAR, WS_SMEAR_LINKS, WS_SMEAR_FX, WS_APE_FX, WS_FX,
   WS_COUNT
 };
 

@@ -591,12 +591,14 @@ static GaussCoef gauss_coef(double c, double lo = 0.0) {
 // L2 run before the next ones start, so that the steps read and write L2.
 constexpr size_t GAUSS_WS_BYTES = 64u << 20;
 
-// workspace for the limbs of the spatial links and the flag of k_spatial_links
-static int4 *spatial_limbs(lqcd_ctx *ctx, int vb, int **bad, int *rc) {
+// workspace for the limbs of the spatial links and the flag of k_spatial_links.  APE and
+// Gaussian smearing have one each (slot): the replays of a captured graph of one are not
+// ordered with calls of the other.
+static int4 *spatial_limbs(lqcd_ctx *ctx, int slot, int vb, int **bad, int *rc) {
   Carver sizing(nullptr);
   sizing.take<int4>((size_t)3 * vb * 288);
   sizing.take<int>(1);
-  void *w = workspace(ctx, WS_SMEAR_FX, sizing.size(), rc);
+  void *w = workspace(ctx, slot, sizing.size(), rc);
   if (!w) return nullptr;
   Carver cv(w);
   int4 *links = cv.take<int4>((size_t)3 * vb * 288);
@@ -611,7 +613,7 @@ static int gauss_fx(lqcd_ctx *ctx, const double2 *U, const double2 *in, double2 
   const int vb = (g.V + 31) / 32;
   int rc = LQCD_OK;
   int *bad = nullptr;
-  int4 *links = spatial_limbs(ctx, vb, &bad, &rc);
+  int4 *links = spatial_limbs(ctx, WS_SMEAR_FX, vb, &bad, &rc);
   *done = false;
   if (!links) return rc;
   const size_t nd = (size_t)4 * vb * 96, ne = (size_t)4 * vb * 32;  // per right-hand side
@@ -684,7 +686,7 @@ extern "C" int lqcd_smear_ape(lqcd_ctx *ctx, double alpha, int n_iter, double *o
   const int vb = (g.V + 31) / 32;
   const FxUse use(ctx, st);
   if (use.ok && n_iter > 0)  // (without the workspace: FP64)
-    links = spatial_limbs(ctx, vb, &bad, &rc);
+    links = spatial_limbs(ctx, WS_APE_FX, vb, &bad, &rc);
   if (links) LQCD_CUDA_TRY(ctx, cudaMemsetAsync(bad, 0, sizeof(int), st));
   for (int it = 0; it < n_iter; ++it) {
     double2 *dst = bufs[it % 2];

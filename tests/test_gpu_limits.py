@@ -63,6 +63,32 @@ def test_streams_share_a_context():
         compare(out)
 
 
+def test_captured_smearing_beside_ape():
+    """Replays of a captured Gaussian smearing beside APE smearing on another stream: the two
+    have no workspace in common."""
+    dims, n = (8, 8, 8, 8), 32
+    with lattice(dims, haar_su3_field(dims, 45), 0.12) as (L, h):
+        src = to_dev(gaussian_spinors(dims, 1, 46).reshape(1, -1, 4, 3)).repeat(n, 1, 1, 1)
+        ref, out = torch.empty_like(src), torch.empty_like(src)
+        L.lqcd_smear_ape(h, 0.5, 2)
+        L.lqcd_smear_gaussian(h, src, ref, alpha=0.5, n_iter=4, normalise=True)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            L.lqcd_smear_gaussian(h, src, out, alpha=0.5, n_iter=4, normalise=True)
+        links = torch.empty(int(np.prod(dims)) * 36, dtype=torch.complex128, device="cuda")
+        one, two = torch.cuda.Stream(), torch.cuda.Stream()
+        for _ in range(4):
+            out.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(one):
+                graph.replay()
+            with torch.cuda.stream(two):
+                L.lqcd_smear_ape(h, 0.5, 2, links)
+            torch.cuda.synchronize()
+            assert torch.equal(out, ref)
+
+
 @pytest.mark.parametrize("dims,n", [((4, 4, 4, 4), 3), ((8, 8, 8, 16), 2)])
 def test_largest_iteration_cap(dims, n):
     """max_iter = 2^31 - 1 ends like any other cap that is not reached: one cluster per pair
