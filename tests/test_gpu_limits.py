@@ -1,5 +1,6 @@
 """Calls at the limits of what the entry points accept: several streams on one context,
-and inputs that are not finite, of extreme size or of very different size within a site."""
+inputs that are not finite, of extreme size or of very different size within a site, and
+more right-hand sides than a workspace takes at a time."""
 import ctypes
 import threading
 
@@ -290,3 +291,31 @@ def test_gradient_nan_coefficient():
         coef[2, 3] = np.nan  # a slice without sources
         _, rc, st = L.lqcd_gradient(h, s, sol, coef, prm, dU=dU)
         assert rc == L.LQCD_ERR_NONFINITE and all(q["status"] == rc for q in st)
+
+
+def test_several_chunks_of_right_hand_sides():
+    """More right-hand sides than the limbs' workspaces take at a time (12 for D and the FP64
+    solver, 3 for smearing on this lattice), with a ragged last chunk: the bits of calls with
+    one right-hand side each."""
+    dims = (12, 12, 12, 24)
+    n, V = 14, int(np.prod(dims))
+    U = eps_su3_field(dims, 0.35, 27)
+    g = torch.Generator(device="cuda").manual_seed(28)
+    x = torch.view_as_complex(torch.randn(n, V, 4, 3, 2, dtype=torch.float64, device="cuda", generator=g))
+    x *= torch.logspace(-3, 3, n, dtype=torch.float64, device="cuda")[:, None, None, None]
+    x[3] = 0.0
+    x[3, 17, 2, 1] = 1.0  # converges at another iteration
+    x[12] = 0.0
+    with lattice(dims, U, 0.115) as (L, h):
+        prm = L.solver_params(tol=1e-6, precision=L.LQCD_PREC_FP64, rhs_block=n)
+        calls = [lambda q, o: L.lqcd_apply_dirac(h, q, o), lambda q, o: L.lqcd_apply_dirac(h, q, o, dagger=True),
+                 lambda q, o: L.lqcd_smear_gaussian(h, q, o, alpha=0.7, n_iter=2),
+                 lambda q, o: L.lqcd_solve_batch(h, q, o, prm)]
+        for f in calls:
+            whole, one = torch.empty_like(x), torch.empty_like(x)
+            st = f(x, whole)
+            sts = [f(x[k:k + 1], one[k:k + 1]) for k in range(n)]
+            assert torch.equal(whole, one)
+            if isinstance(st, tuple):
+                assert st[0] == 0 and st[1] == [s[1][0] for s in sts]
+                assert len({s["iterations"] for s in st[1]}) > 2
