@@ -50,13 +50,13 @@ __host__ __device__ __forceinline__ int4 fx_link_entry(double re, double im) {
 __device__ __forceinline__ int fx_max(int m, double2 v) {
   return max(m, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
 }
-// v 2^(1075 + SH - E) for |v| < 2^(E - 1022), towards zero; flip: bit 31 set negates
-template <int SH> __device__ __forceinline__ long long fx_int(double v, int E, int flip) {
+// v 2^(1075 + SH - E) for |v| < 2^(E - 1022), towards zero
+template <int SH> __device__ __forceinline__ long long fx_int(double v, int E) {
   const int hi = __double2hiint(v), lo = __double2loint(v);
   const int s = min(E - ((hi >> 20) & 0x7ff), 63);
   const unsigned mh = (hi & 0xfffff) | 0x100000;
   const unsigned long long m = (((unsigned long long)__funnelshift_l(lo, mh, SH)) << 32) | ((unsigned)lo << SH);
-  const long long neg = (hi ^ flip) >> 31;
+  const long long neg = hi >> 31;
   return ((long long)(m >> s) ^ neg) - neg;
 }
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return c + (long long)a * b; }

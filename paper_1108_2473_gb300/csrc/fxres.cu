@@ -132,8 +132,8 @@ __global__ void __launch_bounds__(2 * FXR_SITES, 4) k_fx_resid(Geom g, int p_out
       fx_split(acc, ah, al);
       y[h] = fx_mad(ah, kh, 0) + ((fx_mad(al, kh, fx_mad(ah, kl, 0)) + (1ll << 28)) >> 29);
     }
-    const long long re = fx_int<FXF_SH>(bv[k].x, Er, 0) - (Ex > 0 ? xi[0] >> dx : 0) + (Em > 0 ? y[0] >> dy : 0);
-    const long long im = fx_int<FXF_SH>(bv[k].y, Er, 0) - (Ex > 0 ? xi[1] >> dx : 0) + (Em > 0 ? y[1] >> dy : 0);
+    const long long re = fx_int<FXF_SH>(bv[k].x, Er) - (Ex > 0 ? xi[0] >> dx : 0) + (Em > 0 ? y[0] >> dy : 0);
+    const long long im = fx_int<FXF_SH>(bv[k].y, Er) - (Ex > 0 ? xi[1] >> dx : 0) + (Em > 0 ? y[1] >> dy : 0);
     v[k] = make_float2(__ll2float_rn(re) * f.x * f.y, __ll2float_rn(im) * f.x * f.y);
     if (bad) v[k] = make_float2(__int_as_float(0x7fffffff), __int_as_float(0x7fffffff));
     rn = fmaf(v[k].x, v[k].x, fmaf(v[k].y, v[k].y, rn));

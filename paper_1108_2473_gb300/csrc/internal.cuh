@@ -295,6 +295,7 @@ int launch_hop64(lqcd_ctx *ctx, cudaStream_t st, bool dag, bool in_canon, bool o
                  const double2 *B, double cB, double cH, const int *active, int nrhs);
 int fp64_true_residual(lqcd_ctx *ctx, const double2 *b, const double2 *x, int nrhs, double *rr, double *bb,
                        cudaStream_t st);
+int fp64_norms(lqcd_ctx *ctx, const double2 *b, int nrhs, double *bb, cudaStream_t st);
 int fp64_apply_dirac(lqcd_ctx *ctx, const double2 *in, double2 *out, int nrhs, bool dagger,
                      cudaStream_t st);
 int fp64_solve(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs, const lqcd_solver_params &p,

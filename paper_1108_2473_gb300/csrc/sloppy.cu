@@ -291,12 +291,6 @@ __device__ __forceinline__ void hop_dir32n(const Geom &g, int p_out, const int c
   }
 }
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // What a kernel's per-thread sums are: <.,.> alone (in .a, .b of the partial),
 // with a squared norm in .c or in .d, or the norm alone in .c.
 enum { SUM_DOT = 0, SUM_DOT_C = 1, SUM_DOT_D = 2, SUM_NORM = 3 };
@@ -430,7 +424,7 @@ __global__ void __launch_bounds__(ST, EPI == EPI_PLAIN ? 3 : 4) k_hop32x2(Geom g
     const int i = sb * ST + threadIdx.x;
     float2 red = make_float2(0.f, 0.f);  // |out|^2 of the two right-hand sides
     if (i < g.Vh) red = hop32x2_site<EPI>(g, p_out, i, links, in, out, A, B, cA, cB, cH, rhs, two);
-    if (EPI == EPI_RES)  // an odd last entry has only one right-hand side (its second sum is not stored)
+    if (EPI == EPI_RES)  // an odd last entry has only one right-hand side (its second sum is the first again, stored to the same place)
       pair_reduce_store<1, SUM_NORM>(red, red, red, part + (size_t)rhs[0] * nbx + sb,
                                      part + (size_t)rhs[1] * nbx + sb, true);
   }
@@ -2040,9 +2034,6 @@ static int sloppy_alloc(lqcd_ctx *ctx, int nrhs, int gran = 2) {
   return LQCD_OK;
 }
 
-int fp64_residual_into(lqcd_ctx *ctx, const double2 *b, const double2 *x, double2 *res, int nrhs, double *rr,
-                       double *bb, cudaStream_t st);
-
 template <class SP> SP pair_field(SloppyState *st, int f, int vh);
 template <> F16P pair_field<F16P>(SloppyState *st, int f, int vh) {
   size_t pairs = st->cap / 2;
@@ -2334,10 +2325,11 @@ struct MixedRun : RunIface {
       todo = hl;
       for (int k : todo) shift.push_back(-std::ilogb(rr[k]) / 2);
     }
-    int rc = cycle == 0 ? fp64_residual_into(ctx, b, nullptr, nullptr, nrhs, rr.data(), bb.data(), st)
+    int rc = cycle == 0 ? fp64_norms(ctx, b, nrhs, bb.data(), st)
                         : fx_residual(ctx, ss->x, b, res, todo.data(), shift.data(), (int)todo.size(), rr.data(),
                                       st);
     if (rc) return rc;
+    if (cycle == 0) rr = bb;
     if (cycle > 0)  // the scalars that cycle_end asked for came with the residual
       for (int k : todo) hs[k] = host.sc[k];
     hl.clear();
@@ -2561,26 +2553,6 @@ static RunIface *make_run(lqcd_ctx *ctx, const double2 *b, double2 *x, int nrhs,
   if (tuned_code(ctx, nrhs, p.precision) % 10 == TILE_VARIANT)
     return new MixedRun<TileOps>(ctx, b, x, nrhs, p, stats, st, t0);
   return new MixedRun<PairOps<BF16P>>(ctx, b, x, nrhs, p, stats, st, t0);
-}
-
-// capture `body(stream)` into an executable graph on stream st; *kernels
-// receives the number of kernel launches the body recorded (each replay makes
-// them; the capture itself launches nothing, so the library's launch counter
-// is set back)
-template <class F>
-static cudaError_t capture_graph(cudaStream_t st, F body, cudaGraphExec_t *exec, long long *kernels) {
-  cudaGraph_t graph = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return e;
-  const long long before = g_launches.load();
-  body(st);
-  *kernels = g_launches.load() - before;
-  g_launches -= *kernels;
-  e = cudaStreamEndCapture(st, &graph);
-  if (e != cudaSuccess) return e;
-  e = cudaGraphInstantiate(exec, graph, 0);
-  cudaGraphDestroy(graph);
-  return e;
 }
 
 constexpr int ITERS_PER_POLL = 4;  // inner iterations per host poll when launching directly (profiling)
