@@ -63,7 +63,8 @@ typedef struct CUstream_st *lqcd_stream_t; /* same type as cudaStream_t */
 #define LQCD_ERR_OOM (-9)           /* device allocation failed                    */
 
 /* ---- enums ------------------------------------------------------------- */
-#define LQCD_PREC_FP64 0        /* FP64 storage and arithmetic throughout           */
+#define LQCD_PREC_FP64 0        /* FP64 storage and arithmetic; products with SU(3)
+                                   links in 58-bit integers (lqcd_apply_dirac)      */
 #define LQCD_PREC_MIXED_FP16 1  /* FP16 (+ per-site FP32 norm) spinors, FP16 links,
                                    FP32 arithmetic, FP64 defect correction          */
 #define LQCD_PREC_MIXED_BF16 2  /* BF16 spinors, FP16 links, otherwise as above     */
@@ -220,7 +221,13 @@ int lqcd_autotune(lqcd_ctx *ctx, int nrhs, int precision, int *best_blocks_per_s
  * autotuner, any revision by earlier solves and the LQCD_HOP_VARIANT override --
  * as for lqcd_autotune (host ints, each may be NULL; hop variant 5 is the tile
  * layout; an override to variant 6 where it does not apply reports variant 1,
- * the kernel then launched).  Host only; LQCD_ERR_INVALID for a null ctx. */
+ * the kernel then launched).  It is the choice for inner iterations that are
+ * launched.  A small solve in the pair layout, of at most 2048 sites per parity
+ * and few enough right-hand sides for its clusters to run together, makes no
+ * such launches: each pair of right-hand sides is solved by one cluster, to the
+ * same bits as variants 0 to 3, whatever the choice.  With LQCD_HOP_VARIANT or
+ * LQCD_NO_GRAPH set, and while profiling, it is launched like the others.
+ * Host only; LQCD_ERR_INVALID for a null ctx. */
 int lqcd_tuned_choice(const lqcd_ctx *ctx, int nrhs, int precision, int *blocks_per_sm, int *hop_variant);
 
 /* Point sources e_{x,spin,colour} (Sec. II: exact all-to-all propagator from
@@ -301,8 +308,9 @@ int lqcd_smear_ape(lqcd_ctx *ctx, double alpha, int n_iter, double *out, lqcd_st
  * in, out: [nrhs][V][4][3] complex128 device, distinct.  On SU(3) links the
  * steps run in 58-bit integer arithmetic (relative to each site and spin's
  * colour vector; a vector with an entry that is not finite becomes NaN), else
- * in FP64.  Errors: INVALID (in == out, host pointers, ape_links without lqcd_smear_ape),
- * NO_GAUGE. */
+ * in FP64, as for APE links that are not unitary (the projection of a singular
+ * sum is NaN).  Errors: INVALID (in == out, host pointers, ape_links without
+ * lqcd_smear_ape), NO_GAUGE. */
 int lqcd_smear_gaussian(lqcd_ctx *ctx, const double *in, double *out, int nrhs, double alpha, int n_iter,
                         int ape_links, int normalise, lqcd_stream_t stream);
 

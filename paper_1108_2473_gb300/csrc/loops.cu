@@ -178,7 +178,7 @@ __global__ void k_loops_fin(int nbx, const double2 *part, double2 *per_t) {
 static void launch_loops(cudaStream_t st, const Geom &g, const double2 *src, const double2 *sol, int nrhs,
                          double weight, double2 *per_site, double2 *part, int nbx) {
   const int lt = g.L[3];
-  if ((long long)nbx * lt <= 304)
+  if ((long long)nbx * lt <= 2 * 152)
     KL k_loops<4><<<dim3(nbx, lt), 4 * LOOP_THREADS, 0, st>>>(g, src, sol, nrhs, weight, per_site, part);
   else
     KL k_loops<1><<<dim3(nbx, lt), LOOP_THREADS, 0, st>>>(g, src, sol, nrhs, weight, per_site, part);

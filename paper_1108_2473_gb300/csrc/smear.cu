@@ -1,5 +1,6 @@
 // Gaussian quark smearing and APE link smearing (Sec. III, smearing of the
-// interpolating fields), FP64.  These act on the sources of connected
+// interpolating fields): link products in 58-bit integers for SU(3) links, else in
+// FP64, the SU(3) projection in FP64.  These act on the sources of connected
 // correlators; the loops themselves are computed without smearing.
 //
 // Gaussian:  F = (1 + alpha H)^n within each time slice,

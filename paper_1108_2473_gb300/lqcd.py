@@ -477,7 +477,8 @@ def lqcd_batch_destroy(batch):
 
 
 def lqcd_tuned_choice(h, nrhs, precision):
-    """The launch choice later solves of (nrhs, precision) use: (blocks per SM, hop variant)."""
+    """The launch choice of later solves of (nrhs, precision) that launch their inner
+    iterations: (blocks per SM, hop variant)."""
     best = ctypes.c_int(0)
     var = ctypes.c_int(0)
     _check(load().lqcd_tuned_choice(h, int(nrhs), int(precision), ctypes.byref(best), ctypes.byref(var)), h)
