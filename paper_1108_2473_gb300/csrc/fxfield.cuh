@@ -30,6 +30,9 @@ constexpr int FX_ROW_ZERO = 31;
 // largest component, to which all limbs are aligned, are evaluated in FP64: rows 0 and 1 do
 // not mix, so FP64 arithmetic rounds relative to each.  The limbs' rounding is about
 // 2^-55.5 of the stencil's largest component, that of FP64 arithmetic 2^-52.5 of the row's.
+// Error of H against quadruple precision in row 1 of a Gaussian field on 8^4 whose rows 1
+// to 3 are 1, 2^-2, 2^-3, 2^-4 of row 0: 0.7, 0.9, 1.3, 1.5e-16 (2.4e-16 for the last with
+// limbs alone); in FP64 arithmetic 1.55e-16 for all.
 constexpr int FX_ROW_BITS = 3;
 
 __host__ __device__ inline int fx_blocks(int vh) { return (vh + 31) / 32; }
