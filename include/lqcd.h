@@ -128,7 +128,9 @@ const char *lqcd_last_error(const lqcd_ctx *ctx);
  * computed on).  U: [V][4][3][3] complex128, device or host pointer.  Keeps an
  * FP64 copy and the reduced-precision copies the mixed-precision solver reads:
  * FP32 reconstruct-12 (first two rows; the third is (row1 x row2)^*), FP16 with
- * all 18 reals duplicated, tf32 and 58-bit integers.  Errors: LQCD_ERR_NOT_SU3 if
+ * all 18 reals duplicated, tf32 and 58-bit integers, and reserves a workspace for
+ * lqcd_apply_dirac (196 B per site and right-hand side for up to 1024 of them, at
+ * most 96 MiB or one right-hand side).  Errors: LQCD_ERR_NOT_SU3 if
  * a link deviates from unitarity or unit determinant by more than 1e-12
  * (nothing is kept).  NaN entries do not count as a deviation: such a field is
  * kept, FP64 calls then give NaN where the link enters, and solves report
